@@ -186,22 +186,88 @@ __global__ void scatter_kernel(int64_t nmax, const int64_t *d_count, const int32
 
 // compare-exchange network of the "flip" bitonic sort: only ascending
 // exchanges, so values past the segment end behave as +infinity and their
-// exchanges are no-ops.
-__device__ __forceinline__ int warp_sort32(int v)
+// exchanges are no-ops.  A warp sorts 32 K values held in registers, K per
+// lane, element lane * K + k: exchanges at a distance below K stay in the
+// lane, the others are one shuffle each.
+template <int K>
+__device__ __forceinline__ void warp_sort(int (&v)[K])
 {
-    int lane = threadIdx.x & 31;
+    const int lane = threadIdx.x & 31;
 #pragma unroll
-    for (int k = 2; k <= 32; k <<= 1) {
-        int partner = lane ^ (k - 1);
-        int o = __shfl_xor_sync(0xffffffffu, v, k - 1);
-        v = (lane < partner) ? min(v, o) : max(v, o);
+    for (int n = 2; n <= 32 * K; n <<= 1) {
+        // flip: e against e ^ (n - 1)
+        if (n <= K) {
 #pragma unroll
-        for (int j = k >> 2; j > 0; j >>= 1) {
-            int o2 = __shfl_xor_sync(0xffffffffu, v, j);
-            v = ((lane & j) == 0) ? min(v, o2) : max(v, o2);
+            for (int k = 0; k < K; ++k) {
+                const int l = k ^ (n - 1);
+                if (l > k) {
+                    const int a = min(v[k], v[l]), b = max(v[k], v[l]);
+                    v[k] = a;
+                    v[l] = b;
+                }
+            }
+        } else {
+            const int m = n / K - 1;
+            const bool low = (lane & ((m + 1) >> 1)) == 0;
+            int o[K];
+#pragma unroll
+            for (int k = 0; k < K; ++k) o[k] = __shfl_xor_sync(0xffffffffu, v[K - 1 - k], m);
+#pragma unroll
+            for (int k = 0; k < K; ++k) v[k] = low ? min(v[k], o[k]) : max(v[k], o[k]);
+        }
+        // then distances n / 4 .. 1
+#pragma unroll
+        for (int j = n >> 2; j > 0; j >>= 1) {
+            if (j < K) {
+#pragma unroll
+                for (int k = 0; k < K; ++k) {
+                    const int l = k ^ j;
+                    if (l > k) {
+                        const int a = min(v[k], v[l]), b = max(v[k], v[l]);
+                        v[k] = a;
+                        v[l] = b;
+                    }
+                }
+            } else {
+                const bool low = (lane & (j / K)) == 0;
+#pragma unroll
+                for (int k = 0; k < K; ++k) {
+                    const int o = __shfl_xor_sync(0xffffffffu, v[k], j / K);
+                    v[k] = low ? min(v[k], o) : max(v[k], o);
+                }
+            }
         }
     }
-    return v;
+}
+
+// one segment of m <= 32 K indices: read striped, left alone if in order,
+// else sorted in registers, turned to the striped order through shared memory
+// (32 K ints of the warp's own) and written back
+template <int K>
+__device__ __forceinline__ void sort_segment(int32_t *seg, int m, int *s)
+{
+    const unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    int v[K];
+#pragma unroll
+    for (int k = 0; k < K; ++k) v[k] = k * 32 + lane < m ? seg[k * 32 + lane] : INT_MAX;
+    bool ok = true;
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        int next = __shfl_down_sync(FULL, v[k], 1);
+        const int first = k + 1 < K ? __shfl_sync(FULL, v[k + 1 < K ? k + 1 : k], 0) : INT_MAX;
+        if (lane == 31) next = first;
+        ok &= v[k] <= next;
+    }
+    if (__all_sync(FULL, ok)) return;  // the usual case for cells nobody entered
+    warp_sort<K>(v);
+#pragma unroll
+    for (int k = 0; k < K; ++k) s[lane * K + k] = v[k];
+    __syncwarp();
+#pragma unroll
+    for (int k = 0; k < K; ++k)
+        if (k * 32 + lane < m) seg[k * 32 + lane] = s[k * 32 + lane];
+    __syncwarp();
 }
 
 __device__ void smem_sort_warp(int *s, int m)
@@ -231,36 +297,50 @@ __device__ void smem_sort_warp(int *s, int m)
     }
 }
 
+// Bound by the network's instructions, so segments up to 256 (the usual ones:
+// tens of particles per cell) stay in registers; the shared-memory network
+// serves 257 .. SEG_WARP_MAX.  Two steps from a restart (the first sort general)
+// with 4.19e8 particles in 2048^2 cells, 100 to a cell: 57.3 -> 45.4 ms against
+// the network in shared memory for every segment over 32 (12.5 ms of them);
+// 1.68e7 in 512^2: 2.72 -> 2.34 ms.
+// A warp takes `per` consecutive cells, whose starts the lanes hold.
 __global__ void __launch_bounds__(SEG_WARPS * 32) segfix_kernel(const int32_t *offset, int32_t *perm, int ncell,
-                                                                 int32_t *bigseg, int32_t *nbig, const int32_t *flag)
+                                                                 int per, int32_t *bigseg, int32_t *nbig,
+                                                                 const int32_t *flag)
 {
     if (general_off(flag)) return;
     __shared__ int sh[SEG_WARPS][SEG_WARP_MAX];
-    int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (int64_t cellk = (int64_t)blockIdx.x * SEG_WARPS + warp; cellk < ncell;
-         cellk += (int64_t)gridDim.x * SEG_WARPS) {
-        int start = offset[cellk];
-        int m = offset[cellk + 1] - start;
-        if (m <= 1) continue;
-        int32_t *seg = perm + start;
-        // already in order?  (the usual case for cells nobody entered)
-        bool ok = true;
-        for (int i = lane; i + 1 < m; i += 32) ok &= seg[i] <= seg[i + 1];
-        if (__all_sync(0xffffffffu, ok)) continue;
-        if (m <= 32) {
-            int v = lane < m ? seg[lane] : INT_MAX;
-            v = warp_sort32(v);
-            if (lane < m) seg[lane] = v;
-        } else if (m <= SEG_WARP_MAX) {
-            int *s = sh[warp];
-            for (int i = lane; i < m; i += 32) s[i] = seg[i];
-            __syncwarp();
-            smem_sort_warp(s, m);
-            for (int i = lane; i < m; i += 32) seg[i] = s[i];
-            __syncwarp();
-        } else if (lane == 0) {
-            int k = atomicAdd(nbig, 1);
-            bigseg[k] = (int32_t)cellk;
+    const unsigned FULL = 0xffffffffu;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    int *s = sh[warp];
+    const int64_t step = (int64_t)gridDim.x * SEG_WARPS * per;
+    for (int64_t c0 = ((int64_t)blockIdx.x * SEG_WARPS + warp) * per; c0 < ncell; c0 += step) {
+        const int nc = (int)((int64_t)per < ncell - c0 ? (int64_t)per : ncell - c0);
+        const int lo = lane < nc ? offset[c0 + lane] : 0, hi = lane < nc ? offset[c0 + lane + 1] : 0;
+        unsigned todo = __ballot_sync(FULL, hi - lo > 1);
+        while (todo) {
+            const int c = __ffs(todo) - 1;
+            todo &= todo - 1;
+            const int start = __shfl_sync(FULL, lo, c);
+            const int m = __shfl_sync(FULL, hi, c) - start;
+            int32_t *seg = perm + start;
+            if (m <= 32)
+                sort_segment<1>(seg, m, s);
+            else if (m <= 64)
+                sort_segment<2>(seg, m, s);
+            else if (m <= 128)
+                sort_segment<4>(seg, m, s);
+            else if (m <= 256)
+                sort_segment<8>(seg, m, s);
+            else if (m <= SEG_WARP_MAX) {
+                for (int i = lane; i < m; i += 32) s[i] = seg[i];
+                __syncwarp();
+                smem_sort_warp(s, m);
+                for (int i = lane; i < m; i += 32) seg[i] = s[i];
+                __syncwarp();
+            } else if (lane == 0) {
+                bigseg[atomicAdd(nbig, 1)] = (int32_t)(c0 + c);
+            }
         }
     }
 }
@@ -468,6 +548,12 @@ __global__ void __launch_bounds__(256) count9_kernel(const int32_t *off, const i
     }
     const int64_t ntask = ((int64_t)ncell + TASK_CELLS - 1) / TASK_CELLS;
     for (int64_t t = wid; t < ntask; t += nw) {
+        // once a block has found the precondition broken the counts are not
+        // used: the rest of the pass is left out (a restart from another state
+        // then costs one task per warp instead of the whole pass)
+        int broken = 0;
+        if (lane == 0) broken = *(volatile int32_t *)flag;
+        if (__shfl_sync(FULL, broken, 0)) return;
         const int64_t s0 = t * TASK_CELLS;
         const int m = (int)((int64_t)ncell - s0 < TASK_CELLS ? (int64_t)ncell - s0 : TASK_CELLS);
         const int o = off[s0 + (lane < m ? lane : m)];
@@ -672,6 +758,26 @@ cudaError_t launch_keys(grpic_ctx *ctx, const grpic_particles *p, cudaStream_t s
     return cudaGetLastError();
 }
 
+namespace {
+
+// cells per warp: 32 (one coalesced read of the starts) once every resident
+// warp has that many, fewer on small grids so that the work spreads over the
+// SMs (7 blocks of 32 KB shared memory each)
+void launch_segfix(grpic_ctx *ctx, int32_t *nbig, const int32_t *flag, cudaStream_t s)
+{
+    const int64_t ncell = (int64_t)ctx->g.nr * ctx->g.nth;
+    int sms = 152;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device);
+    int per = 1;
+    while (per < 32 && ncell > (int64_t)per * sms * 7 * SEG_WARPS) per <<= 1;
+    const int64_t want = (ncell + (int64_t)per * SEG_WARPS - 1) / ((int64_t)per * SEG_WARPS);
+    const unsigned grid = (unsigned)std::min<int64_t>(want, (int64_t)sms * 64);
+    segfix_kernel<<<grid, SEG_WARPS * 32, 0, s>>>(ctx->d_offset, ctx->d_perm, (int)ncell, per, ctx->d_bigseg, nbig,
+                                                  flag);
+}
+
+}  // namespace
+
 // Expects ctx->d_keys / ctx->d_count filled for the current order of *p.
 cudaError_t launch_sort(grpic_ctx *ctx, grpic_particles *p, grpic_particles *q, cudaStream_t s)
 {
@@ -690,8 +796,7 @@ cudaError_t launch_sort(grpic_ctx *ctx, grpic_particles *p, grpic_particles *q, 
         scatter_kernel<<<blocks, 256, 0, s>>>(p->n, p->d_count, ctx->d_keys, ctx->d_offset, ctx->d_cursor, ctx->d_perm,
                                               ncell, nullptr);
     }
-    segfix_kernel<<<(ncell + SEG_WARPS - 1) / SEG_WARPS, SEG_WARPS * 32, 0, s>>>(ctx->d_offset, ctx->d_perm, ncell,
-                                                                                 ctx->d_bigseg, nbig, nullptr);
+    launch_segfix(ctx, nbig, nullptr, s);
     // oversized segments (rare): the list length is only known on the device,
     // so a fixed grid strides over it and returns at once when it is empty
     bigseg_kernel<<<64, 1024, SEG_BLOCK_MAX * sizeof(int), s>>>(ctx->d_offset, ctx->d_perm, ctx->d_bigseg, nbig,
@@ -782,11 +887,10 @@ cudaError_t launch_sort_step(grpic_ctx *ctx, grpic_particles *p, grpic_particles
     // that skipping them costs little
     const int64_t gmax = (int64_t)dev_sms * 64;
     const unsigned gp = (unsigned)std::max<int64_t>(1, std::min<int64_t>((p->n + 255) / 256, gmax));
-    const unsigned gs = (unsigned)std::max<int64_t>(1, std::min<int64_t>((ncell + SEG_WARPS - 1) / SEG_WARPS, gmax));
     if (p->n > 0)
         scatter_kernel<<<gp, 256, 0, s>>>(p->n, p->d_count, ctx->d_keys, ctx->d_offset, ctx->d_cursor, ctx->d_perm,
                                           ncell, flag);
-    segfix_kernel<<<gs, SEG_WARPS * 32, 0, s>>>(ctx->d_offset, ctx->d_perm, ncell, ctx->d_bigseg, nbig, flag);
+    launch_segfix(ctx, nbig, flag, s);
     bigseg_kernel<<<64, 1024, SEG_BLOCK_MAX * sizeof(int), s>>>(ctx->d_offset, ctx->d_perm, ctx->d_bigseg, nbig, flag);
     GatherArgs G;
     G.nmax = p->n;
