@@ -193,6 +193,13 @@ __host__ __device__ constexpr int tape_width(int n_iter) { return tape_end(n_ite
 
 // entry points implemented in the kernel translation units (host side)
 namespace grpic {
+// SMs of a device (152 if the query fails)
+inline int sm_count(int device)
+{
+    int n = 152;
+    cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, device);
+    return n;
+}
 cudaError_t launch_tables(grpic_ctx *ctx, cudaStream_t s);
 cudaError_t launch_init_fields(grpic_ctx *ctx, int kind, double B0, const grpic_fields *f, cudaStream_t s);
 // push (fused with the deposit) of the particles of `in` into `p`: in place
