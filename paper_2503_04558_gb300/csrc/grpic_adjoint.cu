@@ -475,12 +475,6 @@ __device__ __forceinline__ double W1(double d)
 }
 __device__ __forceinline__ double dW1(double d) { return fabs(d) < 1.0 ? (d > 0.0 ? -1.0 : (d < 0.0 ? 1.0 : 0.0)) : 0.0; }
 
-__device__ __forceinline__ int jcell(const GridDev &g, double x2)
-{
-    int j = (int)floor(x2);
-    return j > g.nth - 1 ? g.nth - 1 : j;
-}
-
 // staggered bilinear stencil with axis mirroring (as in the push)
 struct St {
     int c0, r0, r1;
@@ -578,9 +572,8 @@ __global__ void __launch_bounds__(128) particle_adjoint(PAdjArgs A)
         for (int k = 0; k < 5; ++k) A.lam0[k][p] = 0.0;
         return;
     }
-    double x1a = (log(r) - g.ln_rin) / g.dx1, x2a = th / g.dth;
-    if (x1a >= (double)g.nr) x1a = nextafter((double)g.nr, 0.0);  // as in the push
-    if (x1a < 0.0) x1a = 0.0;
+    const ColPos ca = r_column_in(g, r);  // as in the push
+    const double x1a = ca.i + ca.f, x2a = theta_cells(g, th);
     const double dt = A.dt, eps = massive ? 1.0 : 0.0;
     // the forward push's record: u' after the Boris step, the corrector
     // iterates, x^{n+1} before the reflection
@@ -595,11 +588,12 @@ __global__ void __launch_bounds__(128) particle_adjoint(PAdjArgs A)
     double th1 = y1[1];
     if (th1 < 0.0) { th1 = -th1; refl = -1.0; }
     else if (th1 > M_PI) { th1 = 2.0 * M_PI - th1; refl = -1.0; }
-    double x1b = (log(y1[0]) - g.ln_rin) / g.dx1, x2b = th1 / g.dth;
-    int i0 = (int)floor(x1a), j0 = jcell(g, x2a);
-    int di = (int)floor(x1b) - i0, dj = jcell(g, x2b) - j0;
+    const ColPos cb = r_column(g, y1[0]);
+    const double x1b = cb.i + cb.f, x2b = theta_cells(g, th1);
+    const int i0 = ca.i, j0 = row_of(g, x2a);
+    const int di = cb.i - i0, dj = row_of(g, x2b) - j0;
     // the push's own checks: a finite end point, at most one cell away
-    bool moved_ok = di >= -1 && di <= 1 && dj >= -1 && dj <= 1 && isfinite(x1b) && isfinite(x2b) &&
+    bool moved_ok = di >= -1 && di <= 1 && dj >= -1 && dj <= 1 && y1[0] > 0.0 && isfinite(y1[0]) && isfinite(x2b) &&
                     isfinite(y1[2]) && isfinite(y1[3]) && isfinite(dphi);
     if (!moved_ok) {
         for (int k = 0; k < 5; ++k) A.lam0[k][p] = 0.0;

@@ -59,6 +59,47 @@ void gauss_legendre(int n, double *x, double *w)
     }
 }
 
+// GridDev's tables and series for cells and sin, cos without the library's
+// functions (FP64 contexts).  The series runs to the term below 2^-54 of a cell
+// half a cell (and the guess's error) from the centre, at most CELL_TERMS: cells up
+// to dx1 = 0.18; from dx1 = 1e-4 the FP32 guess is within a few hundredths of a
+// column.  Rows up to 0.05 rad (n_theta >= 63) for the shift's series.
+cudaError_t cell_tables(grpic_ctx *ctx)
+{
+    GridDev &g = ctx->g;
+    const double y = std::exp(0.53 * g.dx1) - 1.0;
+    int n = 1;
+    while (n <= CELL_TERMS && std::pow(y, n + 1) / ((n + 1) * g.dx1) > 5e-17) ++n;
+    cudaError_t e = cudaSuccess;
+    if (n <= CELL_TERMS && g.dx1 >= 1e-4) {
+        g.nser = n;
+        for (int k = 0; k < n; ++k) g.cser[k] = ((k & 1) ? -1.0 : 1.0) / ((k + 1) * g.dx1);
+        g.ln_rinf = (float)g.ln_rin;
+        g.idx1f = (float)(1.0 / g.dx1);
+        std::vector<double2> h(g.ld_tab);
+        for (int c = 0; c < g.ld_tab; ++c) {
+            // (rounded once: a centre's error is an error of every offset in its column)
+            const double r = (double)(g.r_in * std::exp((c - NG + 0.5L) * (long double)g.dx1));
+            h[c] = make_double2(r, 1.0 / r);
+        }
+        e = cudaMalloc(&ctx->rcen, sizeof(double2) * h.size());
+        if (e == cudaSuccess) e = cudaMemcpy(ctx->rcen, h.data(), sizeof(double2) * h.size(), cudaMemcpyHostToDevice);
+        g.rcen = ctx->rcen;
+    }
+    if (e == cudaSuccess && g.dth <= 0.05) {
+        std::vector<double2> h(2 * (size_t)(g.nth + 1));
+        for (int j = 0; j <= g.nth; ++j) {
+            const double t = j * g.dth;
+            h[2 * j] = make_double2(t, std::sin(t));
+            h[2 * j + 1] = make_double2(std::cos(t), 0.0);
+        }
+        e = cudaMalloc(&ctx->trow, sizeof(double2) * h.size());
+        if (e == cudaSuccess) e = cudaMemcpy(ctx->trow, h.data(), sizeof(double2) * h.size(), cudaMemcpyHostToDevice);
+        g.trow = ctx->trow;
+    }
+    return e;
+}
+
 __global__ void to_float(const double *a, float *b, size_t n)
 {
     size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -357,6 +398,7 @@ grpic_status grpic_init(grpic_metric metric, double spin, const grpic_grid *grid
     g.dx1 = std::log(grid->r_out / grid->r_in) / grid->n_r;
     g.dth = M_PI / grid->n_theta;
     g.ln_rin = std::log(grid->r_in);
+    g.idth = 1.0 / g.dth;
     gauss_legendre(NGL, ctx->gl_x, ctx->gl_w);
     ctx->slab = (size_t)(g.nth + 1) * g.ld_tab;
     int64_t ncell = (int64_t)g.nr * g.nth;
@@ -374,6 +416,7 @@ grpic_status grpic_init(grpic_metric metric, double spin, const grpic_grid *grid
     if (e == cudaSuccess) e = cudaMalloc(&ctx->d_cnt9, sizeof(int32_t) * 9 * ncell);
     if (e == cudaSuccess) e = cudaMalloc(&ctx->d_base9, sizeof(int32_t) * 9 * ncell);
     if (e == cudaSuccess) e = cudaMalloc(&ctx->d_sortflag, sizeof(int32_t));
+    if (e == cudaSuccess && prm->precision == 64) e = cell_tables(ctx);
     if (e == cudaSuccess) {
         e = cudaMalloc(&ctx->rcol, sizeof(double) * g.ld_tab);
         if (e == cudaSuccess) {
@@ -393,12 +436,6 @@ grpic_status grpic_init(grpic_metric metric, double spin, const grpic_grid *grid
     cudaMemcpy((char *)ctx->d_status + 16, prm->q_weight, 4 * sizeof(double), cudaMemcpyHostToDevice);
     e = launch_tables(ctx, 0);
     if (e == cudaSuccess) e = sort_setup();
-    if (e == cudaSuccess && (prm->radiation || prm->injection)) {
-        e = cudaMalloc(&ctx->d_spqm, 4 * sizeof(double));
-        if (e == cudaSuccess) e = cudaMalloc(&ctx->d_spmassive, 4 * sizeof(int));
-        if (e == cudaSuccess) e = cudaMemcpy(ctx->d_spqm, prm->q_over_m, 4 * sizeof(double), cudaMemcpyHostToDevice);
-        if (e == cudaSuccess) e = cudaMemcpy(ctx->d_spmassive, prm->massive, 4 * sizeof(int), cudaMemcpyHostToDevice);
-    }
     if (e == cudaSuccess && prm->precision == 32) {
         e = cudaMalloc(&ctx->tab32, sizeof(float) * ctx->slab * T_COUNT);
         if (e == cudaSuccess) e = cudaMalloc(&ctx->col1d32, sizeof(float) * 4 * g.ld_tab);
@@ -1179,7 +1216,7 @@ void grpic_destroy(grpic_ctx *ctx)
     if (ctx->up_stream) cudaStreamDestroy(ctx->up_stream);
     if (ctx->down_stream) cudaStreamDestroy(ctx->down_stream);
     if (ctx->h_count) cudaFreeHost(ctx->h_count);
-    void *ptrs[] = {ctx->d_spawn, ctx->d_rad, ctx->d_spqm, ctx->d_spmassive, ctx->d_offset_prev, ctx->d_cnt9, ctx->d_base9, ctx->d_sortflag, ctx->rcol, ctx->rcol2, ctx->rowsc, ctx->tab, ctx->col1d, ctx->tab32, ctx->col1d32, ctx->fscratch, ctx->q32, ctx->d_status, ctx->d_keys,
+    void *ptrs[] = {ctx->d_spawn, ctx->d_rad, ctx->d_offset_prev, ctx->d_cnt9, ctx->d_base9, ctx->d_sortflag, ctx->rcol, ctx->rcen, ctx->trow, ctx->rcol2, ctx->rowsc, ctx->tab, ctx->col1d, ctx->tab32, ctx->col1d32, ctx->fscratch, ctx->q32, ctx->d_status, ctx->d_keys,
                     ctx->d_count, ctx->d_offset, ctx->d_cursor, ctx->d_blocksum, ctx->d_perm, ctx->d_bigseg};
     for (void *q : ptrs)
         if (q) cudaFree(q);

@@ -172,7 +172,8 @@ __global__ void deposit_kernel(GridDev g, int64_t nmax, const void *xa1, const v
     double q = qw[t & 3u];
     if (shape == 3) {
         if constexpr (sizeof(T) == 8)
-            deposit3(g.nr, g.nth, ld, (double *)J0, (double *)J1, (double *)J2, q, dt, x1a, x2a, x1b, x2b, dp);
+            deposit3(g.nr, g.nth, ld, (double *)J0, (double *)J1, (double *)J2, -0.5 * q / dt, q / dt, i0, x1a - i0,
+                     j0, x2a - j0, i0 + di, x1b - (i0 + di), j0 + dj, x2b - (j0 + dj), dp);
         return;
     }
     double S0r[4], S1r[4], S0t[4], S1t[4];

@@ -28,26 +28,36 @@ struct RhsT {
 // approximations with a relative error of a few ulp for reciprocal and square
 // root; sin/cos keep the accurate sincosf because near the polar axis
 // sin(theta) needs relative accuracy (the fast __sincosf has an absolute error
-// of ~2^-21).  FP64 (the FP64 island of the FP32 form): reciprocal and square
-// root from an FP32 seed refined by two Newton steps in FP64 (relative error
-// below 2^-52 for the normal range used here), sin/cos from the library.
+// of ~2^-21).  FP64: reciprocal and reciprocal square root from the hardware's
+// 20-bit FP64 seeds (rcp / rsqrt.approx.ftz.f64, off the FP64 pipe and without
+// conversions) and one step of third order in the residual e: with 1/x = y0 / (1
+// - e), 1 + e + e^2 leaves e^3, and 1/sqrt(x) = y0 (1 - e)^-1/2, 1 + e/2 + 3 e^2/8
+// leaves 5 e^3 / 16, both below 2^-58.  Measured over exp(-60) .. exp(60): within
+// 1.0 and 1.25 x 2^-53 of the exact value (IEEE division 1.0, 1 / sqrt 1.5); 3
+// and 5 pipe slots, 8 and 10 with FP32 seeds and two Newton steps.  sin/cos from
+// the library.
 __device__ __forceinline__ void sincos_t(double x, double *s, double *c) { sincos(x, s, c); }
 __device__ __forceinline__ void sincos_t(float x, float *s, float *c) { sincosf(x, s, c); }
 __device__ __forceinline__ double rcp_t(double x)
 {
-    double y = (double)__frcp_rn((float)x);
-    y = y * (2.0 - x * y);
-    return y * (2.0 - x * y);
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double e = fma(-x, y, 1.0);
+    return fma(y, fma(e, e, e), y);
+}
+__device__ __forceinline__ double rsqrt_t(double x)
+{
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double e = fma(-x * y, y, 1.0);
+    return fma(y * e, fma(e, 0.375, 0.5), y);
 }
 __device__ __forceinline__ float rcp_t(float x) { return __fdividef(1.0f, x); }
 __device__ __forceinline__ double sqrt_t(double x)
 {
     if (!(x > 0.0)) return 0.0;
-    double y = (double)rsqrtf((float)x);       // 1/sqrt(x), 2^-22
-    y = y * (1.5 - 0.5 * x * y * y);           // 2^-44
-    y = y * (1.5 - 0.5 * x * y * y);           // full precision
-    double s = x * y;
-    return s + 0.5 * y * (x - s * s);          // one correction of the root itself
+    const double y = rsqrt_t(x), s = x * y;
+    return fma(0.5 * y, fma(-s, s, x), s);  // one correction of the root itself
 }
 __device__ __forceinline__ float sqrt_t(float x) { return x > 0.0f ? x * rsqrtf(x) : 0.0f; }
 
@@ -55,13 +65,20 @@ __device__ __forceinline__ float sqrt_t(float x) { return x > 0.0f ? x * rsqrtf(
 // of sin d, cos d; for |d| <= 0.05 the truncated terms are below 1e-17 in
 // FP64 and below 3e-12 (to d^5 and d^4) in FP32.
 template <typename T>
-__device__ __forceinline__ void sincos_shift(T s0, T c0, T d, T &s, T &c)
+__device__ __forceinline__ void sincos_shift(T s0, T c0, T d, T &s, T &c);
+template <>
+__device__ __forceinline__ void sincos_shift<double>(double s0, double c0, double d, double &s, double &c)
 {
-    T d2 = d * d;
-    T sd = d * (T(1) - d2 * (T(1) / T(6)) * (T(1) - d2 * (T(1) / T(20)) * (T(1) - d2 * (T(1) / T(42)))));
-    T cd = T(1) - d2 * T(0.5) * (T(1) - d2 * (T(1) / T(12)) * (T(1) - d2 * (T(1) / T(30)) * (T(1) - d2 * (T(1) / T(56)))));
-    s = s0 * cd + c0 * sd;
-    c = c0 * cd - s0 * sd;
+    const double d2 = d * d;
+    double ps = 1.0 / 120.0, pc = 1.0 / 24.0;
+    // |d| >= 2^-8: two terms more each (below it they are under 5e-18)
+    if ((__double2hiint(d) & 0x7fffffff) >= 0x3f700000) {
+        ps = fma(d2, -1.0 / 5040.0, ps);
+        pc = fma(d2, fma(d2, 1.0 / 40320.0, -1.0 / 720.0), pc);
+    }
+    const double sd = fma(d * d2, fma(d2, ps, -1.0 / 6.0), d), cm = d2 * fma(d2, pc, -0.5);  // sin d, cos d - 1
+    s = fma(c0, sd, fma(s0, cm, s0));
+    c = fma(-s0, sd, fma(c0, cm, c0));
 }
 template <>
 __device__ __forceinline__ void sincos_shift<float>(float s0, float c0, float d, float &s, float &c)
@@ -156,21 +173,12 @@ __device__ __forceinline__ void geo_rhs_m(const KSGeo<M> &m, T eps, T ur, T ut, 
 // (d_th sin^-2 = -2 sin cos / sin^4).  1/(1+z) lies in (0, 1].
 //
 // Per type: the reciprocal and reciprocal square root the right-hand side
-// takes (FP32: the hardware approximations; FP64: an FP32 seed refined by
-// two Newton steps, the residual formed by a fused multiply-add, relative
-// error a few ulp of FP64; arguments within FP32's normal range) and the
-// fused multiply-add
+// takes (FP32: the hardware approximations; FP64: rcp_t, rsqrt_t) and the fused
+// multiply-add
 __device__ __forceinline__ float rcp_fast(float x) { return __fdividef(1.0f, x); }
 __device__ __forceinline__ double rcp_fast(double x) { return rcp_t(x); }
 __device__ __forceinline__ float rsqrt_fast(float x) { return rsqrtf(x); }
-__device__ __forceinline__ double rsqrt_fast(double x)
-{
-    double y = (double)rsqrtf((float)x);  // 2^-22
-    double e = fma(-x * y, y, 1.0);       // 1 - x y^2
-    y = fma(0.5 * y, e, y);               // 2^-43
-    e = fma(-x * y, y, 1.0);
-    return fma(0.5 * y, e, y);
-}
+__device__ __forceinline__ double rsqrt_fast(double x) { return rsqrt_t(x); }
 __device__ __forceinline__ float fmat(float a, float b, float c) { return fmaf(a, b, c); }
 __device__ __forceinline__ double fmat(double a, double b, double c) { return fma(a, b, c); }
 
@@ -180,6 +188,9 @@ struct PtT {
 };
 using Pt32 = PtT<float>;
 
+// FP64 keeps 1 / (1 + z) by a reciprocal (3 pipe slots against a root's 5 and a
+// square) and takes 1 / u^0 = alpha / sqrt(Q) as one root of (1 + z) Q; alpha
+// itself is formed where the Boris step needs it (lapse()).
 template <typename T>
 __device__ __forceinline__ PtT<T> pointT(T a2, T m2a2, T r, T s, T c)
 {
@@ -190,8 +201,13 @@ __device__ __forceinline__ PtT<T> pointT(T a2, T m2a2, T r, T s, T c)
     m.ir = rcp_fast(m.rho2);
     m.z = (r + r) * m.ir;
     m.opz = T(1) + m.z;
-    m.al = rsqrt_fast(m.opz);
-    m.iopz = m.al * m.al;
+    if constexpr (sizeof(T) == 4) {
+        m.al = rsqrt_fast(m.opz);
+        m.iopz = m.al * m.al;
+    } else {
+        m.iopz = rcp_fast(m.opz);
+        m.al = T(0);
+    }
     m.beta = m.z * m.iopz;
     m.s2 = s * s;
     m.is2 = rcp_fast(m.s2);
@@ -200,6 +216,7 @@ __device__ __forceinline__ PtT<T> pointT(T a2, T m2a2, T r, T s, T c)
     m.E = m2a2 * m.cs * m.ir;  // m2a2 = -2 a^2
     return m;
 }
+__device__ __forceinline__ double lapse(const PtT<double> &m) { return rsqrt_fast(m.opz); }
 
 __device__ __forceinline__ Pt32 point32(float a2, float m2a2, float r, float s, float c)
 {
@@ -217,8 +234,11 @@ __device__ __forceinline__ void rhsT(const PtT<T> &m, T a, T eps, T ur, T ut, T 
     const T P = fmat(ur, w + aup, fmat(ut, ut, is2up2));
     const T irP = m.ir * P;
     const T Q = fmat(m.ir, P, fmat(-m.beta, ur2, eps));
-    const T qq = rsqrt_fast(Q);
-    const T iu0 = m.al * qq;                                   // 1 / u^0
+    T iu0;                                                     // 1 / u^0
+    if constexpr (sizeof(T) == 4)
+        iu0 = m.al * rsqrt_fast(Q);
+    else
+        iu0 = rsqrt_fast(m.opz * Q);
     const T h = T(0.5) * iu0;
     const T iri = m.ir * iu0;
     f.xr = fmat(iu0, fmat(m.ir, w, -m.beta * ur), -m.beta);

@@ -9,6 +9,7 @@
 
 #include <vector>
 
+#include <climits>
 #include <cmath>
 #include <cstdint>
 #include <cuda_runtime.h>
@@ -34,9 +35,23 @@ enum TabSlot {
     T_COUNT
 };
 
+constexpr int CELL_TERMS = 16;  // terms of the cell offset's series at most
+
 struct GridDev {
     int nr, nth, ld_tab;
     double a, r_in, r_out, dx1, dth, ln_rin;
+    double idth;  // 1 / dth
+    // FP64 contexts: where a particle's cell and its sin, cos come from without
+    // the library's logarithm and sin / cos.  rcen: centre r_{i+1/2} of every
+    // column (index i + NG) and its inverse; the offset in the cell is
+    // 1/2 + y (cser[0] + y (cser[1] + ...)), y = r / r_{i+1/2} - 1, nser terms (the
+    // series of log(1 + y) / dx1).  trow: theta_j, sin, cos (and a pad) of row j.
+    // nullptr where the cells are too wide (or too narrow for an FP32 guess of
+    // the column) and in contexts without tables: the library functions then.
+    const double2 *rcen, *trow;
+    int nser;
+    float ln_rinf, idx1f;
+    double cser[CELL_TERMS];
 };
 
 }  // namespace grpic
@@ -53,6 +68,7 @@ struct grpic_ctx {
     float *tab32;       // FP32 copies of tab (precision 32 only)
     float *col1d32;
     size_t slab;        // elements per slab = (nth+1)*ld_tab
+    double2 *rcen, *trow;  // GridDev's tables (precision 64 only)
     double *rcol;       // r at integer columns r_in exp(i dx1), index i + NG
     float *rcol2;       // the same as (hi, lo) float pairs (precision 32 only)
     float *rowsc;       // sin, cos of theta_j = j dtheta as (hi, lo) pairs, j = 0..nth (precision 32)
@@ -81,12 +97,9 @@ struct grpic_ctx {
     const uint32_t *pending_tag;
     int counts_ready;  // the last (permuted) push filled d_cnt9 for the next sort
     // 2D radiation and injection: per-slot spawn counts, block sums/offsets,
-    // charged particles and injection flags per cell; q/m and massive per
-    // species on the device
+    // charged particles and injection flags per cell
     int32_t *d_spawn, *d_rad;
     int64_t rad_cap;
-    double *d_spqm;
-    int *d_spmassive;
     int64_t perm_cap;
     int keys_valid;       // keys of the current order are valid
     int hist_valid;       // and so is their histogram (d_count)
@@ -173,6 +186,89 @@ __host__ __device__ inline double ks_sqrtg(double a, double r, double th)
 }
 
 __host__ __device__ inline double r_of(const GridDev &g, double x1) { return g.r_in * exp(x1 * g.dx1); }
+
+// ---------------------------------------------------------------------------
+// FP64 pieces that keep off the FP64 pipe, which issues one warp instruction
+// in about 18 cycles and takes conversions to and from FP32 and integers,
+// comparisons and finiteness tests at the same price.
+// ---------------------------------------------------------------------------
+// a positive normal double cut to 24 bits (exponents within float's range)
+__device__ __forceinline__ float float_of_pos(double x)
+{
+    return __uint_as_float(__funnelshift_l((unsigned)__double2loint(x), (unsigned)__double2hiint(x), 3) - 0xC0000000u);
+}
+__device__ __forceinline__ bool finite64(double x) { return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000; }
+__device__ __forceinline__ bool negative64(double x) { return __double2hiint(x) < 0; }
+__device__ __forceinline__ bool zero64(double x) { return ((__double2hiint(x) << 1) | __double2loint(x)) == 0; }
+// |x| < lim up to the low word (hi_lim: the high word of lim)
+__device__ __forceinline__ bool below64(double x, int hi_lim) { return (__double2hiint(x) & 0x7fffffff) < hi_lim; }
+__device__ __forceinline__ double flip_sign(double x, bool flip)
+{
+    return __hiloint2double(__double2hiint(x) ^ (flip ? 0x80000000 : 0), __double2loint(x));
+}
+
+// theta / dth, correctly rounded (Markstein's division by a rounded inverse)
+__device__ __forceinline__ double theta_cells(const GridDev &g, double th)
+{
+    const double q = th * g.idth;
+    return fma(fma(-q, g.dth, th), g.idth, q);
+}
+
+// row of theta / dth (theta = pi belongs to the last one)
+__device__ __forceinline__ int row_of(const GridDev &g, double x2)
+{
+    const int j = __double2int_rd(x2);
+    return j > g.nth - 1 ? g.nth - 1 : j;
+}
+
+// Column of r > 0 and the offset in it (0 <= f < 1); columns more than NG beyond
+// the grid are reported with an offset of 1/2.  The one definition of a
+// particle's column for the push, the sort's keys, the appended particles and
+// the adjoint: an FP32 logarithm guesses the column, the series in y gives the
+// offset to a few 1e-16 relative to r (the 30-instruction FP64 logarithm and its
+// division: 40 pipe slots against about 10), and one step to the neighbour
+// column mends a guess next to an edge.
+struct ColPos {
+    int i;
+    double f;
+};
+__device__ __forceinline__ ColPos r_column(const GridDev &g, double r)
+{
+    ColPos c;
+    if (g.rcen) {
+        const int e = (int)floorf((__logf(float_of_pos(r)) - g.ln_rinf) * g.idx1f);
+        c.i = e;
+        c.f = 0.5;
+        if (e >= -NG && e < g.nr + NG) {
+            const double2 t = __ldg(g.rcen + (e + NG));
+            const double y = (r - t.x) * t.y;
+            if (!below64(y, 0x3fd00000)) {  // (a value no FP32 guess fits)
+                c.i = INT_MIN / 2;
+                return c;
+            }
+            double s = g.cser[g.nser - 1];
+            for (int k = g.nser - 2; k >= 0; --k) s = fma(s, y, g.cser[k]);
+            const double f = fma(s, y, 0.5);
+            const bool lo = negative64(f), hi = __double2hiint(f) >= 0x3ff00000;
+            c.i = e + (hi ? 1 : 0) - (lo ? 1 : 0);
+            c.f = f + (lo ? 1.0 : (hi && !lo ? -1.0 : 0.0));
+            if (__double2hiint(c.f) >= 0x3ff00000) c.f = 0x1.fffffffffffffp-1;  // -1e-17 + 1
+        }
+    } else {
+        const double x = (log(r) - g.ln_rin) / g.dx1, fl = floor(x);
+        c.i = fl > -1e9 && fl < 1e9 ? (int)fl : INT_MIN / 2;
+        c.f = x - fl;
+    }
+    return c;
+}
+// the column a push starts from: r in [r_in, r_out), rounding clamped into the grid
+__device__ __forceinline__ ColPos r_column_in(const GridDev &g, double r)
+{
+    ColPos c = r_column(g, r);
+    if (c.i < 0) c = {0, 0.0};
+    if (c.i > g.nr - 1) c = {g.nr - 1, 0x1.fffffffffffffp-1};
+    return c;
+}
 
 __device__ inline void set_status(int *st, int code) { atomicCAS(st, 0, code); }
 

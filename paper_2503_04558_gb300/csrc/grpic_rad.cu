@@ -32,17 +32,9 @@ namespace {
 constexpr int RB = 1024;  // slots (or cells) per block of the ordered appends
 constexpr int RT = 256;   // threads per block: four slots each
 
-__device__ __forceinline__ int jcl(const GridDev &g, double x2)
-{
-    int j = (int)floor(x2);
-    return j > g.nth - 1 ? g.nth - 1 : j;
-}
-
 __device__ __forceinline__ int key_of(const GridDev &g, double r, double th)
 {
-    int i = (int)floor((log(r) - g.ln_rin) / g.dx1);
-    i = i < 0 ? 0 : (i > g.nr - 1 ? g.nr - 1 : i);
-    return jcl(g, th / g.dth) * g.nr + i;
+    return row_of(g, theta_cells(g, th)) * g.nr + r_column_in(g, r).i;
 }
 
 // block-exclusive scan of 4 values per thread (slot order = thread-major
@@ -173,22 +165,19 @@ __global__ void count_add(int64_t *d_count, const int32_t *total, int per, int64
     *d_count = v > cap ? cap : v;
 }
 
-// charged live particles per cell
-__global__ void charged_per_cell(GridDev g, const int64_t *d_count, int64_t nmax, const double *r, const double *th,
-                                 const uint32_t *tag, const double *qm, const int *massive, int32_t *nq)
+// charged live particles per cell, by the keys that the push and the appends
+// left for every slot (dead slots: n_cells)
+__global__ void charged_per_cell(int ncell, const int64_t *d_count, int64_t nmax, const int32_t *keys,
+                                 const uint32_t *tag, unsigned charged, int32_t *nq)
 {
     int64_t n = *d_count;
     if (n > nmax) n = nmax;
     const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= n) return;
     const uint32_t t = tag[p];
-    if (t & DEAD) return;
-    const int sp = t & 3u;
-    if (!(massive[sp] && qm[sp] != 0.0)) return;
-    const double x1 = (log(r[p]) - g.ln_rin) / g.dx1;
-    const int i = (int)floor(x1), j = jcl(g, th[p] / g.dth);
-    if (i < 0 || i >= g.nr || j < 0) return;
-    atomicAdd(nq + (size_t)j * g.nr + i, 1);
+    const int key = keys[p];
+    if ((t & DEAD) || !((charged >> (t & 3u)) & 1u) || (unsigned)key >= (unsigned)ncell) return;
+    atomicAdd(nq + key, 1);
 }
 
 // bilinear field at logical (x1, x2) on a lattice staggered by sr (half rows
@@ -232,7 +221,7 @@ __global__ void inject_flags(InjArgs A)
     const double x1 = i + 0.5, x2 = j + 0.5;
     double Dv[3], Bv[3];
     if (A.shape == 3) {
-        gather3_fields(A.D0, A.D1, A.D2, A.B0, A.B1, A.B2, A.ld, A.g.nth, x1, x2, Dv, Bv);
+        gather3_fields(A.D0, A.D1, A.D2, A.B0, A.B1, A.B2, A.ld, A.g.nth, i, 0.5, j, 0.5, Dv, Bv);
     } else {
         Dv[0] = cic_at(A.D0, A.ld, A.g.nth, x1, x2, 0.5, false, 1.0);
         Dv[1] = cic_at(A.D1, A.ld, A.g.nth, x1, x2, 0.0, true, -1.0);
@@ -356,8 +345,10 @@ cudaError_t launch_injection(grpic_ctx *ctx, grpic_particles *p, const grpic_fie
     int32_t *nq = cboff + (nbc + 1), *flag = nq + ncell;
     cudaMemsetAsync(nq, 0, sizeof(int32_t) * (size_t)ncell, s);
     const unsigned gp = (unsigned)((p->capacity + 255) / 256);
-    charged_per_cell<<<gp, 256, 0, s>>>(ctx->g, p->d_count, p->capacity, (const double *)p->x1,
-                                        (const double *)p->x2, p->tag, ctx->d_spqm, ctx->d_spmassive, nq);
+    unsigned charged = 0;
+    for (int k = 0; k < 4; ++k)
+        if (ctx->prm.massive[k] && ctx->prm.q_over_m[k] != 0.0) charged |= 1u << k;
+    charged_per_cell<<<gp, 256, 0, s>>>((int)ncell, p->d_count, p->capacity, ctx->d_keys, p->tag, charged, nq);
     InjArgs I;
     I.g = ctx->g;
     I.D0 = (const double *)f->D[0];

@@ -138,12 +138,9 @@ __global__ void keys_kernel(GridDev g, int64_t nmax, const int64_t *d_count, con
             if (FP64) {
                 double r = ((const double *)x1)[p], th = ((const double *)x2)[p];
                 if (r >= g.r_in && r < g.r_out && th >= 0.0 && th <= M_PI) {
-                    // the cell the push would start from (x1 clamped into [0, nr))
-                    int i = (int)floor((log(r) - g.ln_rin) / g.dx1);
-                    i = i < 0 ? 0 : (i > g.nr - 1 ? g.nr - 1 : i);
-                    int j = (int)floor(th / g.dth);
-                    if (j > g.nth - 1) j = g.nth - 1;
-                    key = j * g.nr + i;
+                    // the cell the push would start from
+                    const int i = r_column_in(g, r).i;
+                    key = row_of(g, theta_cells(g, th)) * g.nr + i;
                 }
             } else {
                 int c = cell[p];

@@ -15,6 +15,8 @@
 // triad (the step uses only dot and cross products).
 #pragma once
 
+#include "grpic_geo.cuh"
+
 namespace grpic {
 
 // metric quantities at the particle: lapse, gamma_ij, gamma^ij, sqrt(gamma)
@@ -24,14 +26,21 @@ struct VayMetric {
     T alpha, g_rr, g_rp, g_tt, g_pp, gi_rr, gi_rp, gi_tt, gi_pp, sqrtg;
 };
 
+// per type: 1 / sqrt(x), sqrt(x) and 1 / x (FP32: IEEE; FP64: the seeded forms)
+__device__ __forceinline__ float vay_rsqrt(float x) { return 1.0f / sqrtf(x); }
+__device__ __forceinline__ float vay_sqrt(float x) { return sqrtf(x); }
+__device__ __forceinline__ float vay_rcp(float x) { return 1.0f / x; }
+__device__ __forceinline__ double vay_rsqrt(double x) { return rsqrt_t(x); }
+__device__ __forceinline__ double vay_sqrt(double x) { return x * rsqrt_t(x); }
+__device__ __forceinline__ double vay_rcp(double x) { return rcp_t(x); }
+
 template <typename T>
 __device__ __forceinline__ void vay_step(const VayMetric<T> &m, T qm, T dt, const T D[3], const T B[3], T u[3])
 {
     // E_i = gamma_ij D^j;  v^j = gamma^jl u_l / Gamma
     const T E0 = m.g_rr * D[0] + m.g_rp * D[2], E1 = m.g_tt * D[1], E2 = m.g_rp * D[0] + m.g_pp * D[2];
     const T w0 = m.gi_rr * u[0] + m.gi_rp * u[2], w1 = m.gi_tt * u[1], w2 = m.gi_rp * u[0] + m.gi_pp * u[2];
-    const T G = sqrt(T(1) + u[0] * w0 + u[1] * w1 + u[2] * w2);
-    const T iG = T(1) / G;
+    const T iG = vay_rsqrt(T(1) + u[0] * w0 + u[1] * w1 + u[2] * w2);
     const T h = qm * m.alpha * dt;
     const T hs = T(0.5) * h * m.sqrtg * iG;
     // u'_i = u_i + h E_i + (h / 2) e_ijk v^j B^k
@@ -45,9 +54,8 @@ __device__ __forceinline__ void vay_step(const VayMetric<T> &m, T qm, T dt, cons
     const T us = p0 * t0 + p1 * t1 + p2 * t2;
     const T q0 = m.gi_rr * p0 + m.gi_rp * p2, q1 = m.gi_tt * p1, q2 = m.gi_rp * p0 + m.gi_pp * p2;
     const T sigma = T(1) + p0 * q0 + p1 * q1 + p2 * q2 - tt;
-    const T G1 = sqrt(T(0.5) * (sigma + sqrt(sigma * sigma + T(4) * (tt + us * us))));
-    const T iG1 = T(1) / G1;
-    const T s = T(1) / (T(1) + tt * iG1 * iG1);
+    const T iG1 = vay_rsqrt(T(0.5) * (sigma + vay_sqrt(sigma * sigma + T(4) * (tt + us * us))));
+    const T s = vay_rcp(T(1) + tt * iG1 * iG1);
     // u1_i = s (u'_i + (u'.t) t_i + e_ijk u'^j t^k), t = tau / Gamma1
     const T ut = us * iG1 * iG1;        // (u'.t) with t_i = tl_i / Gamma1
     const T cs = m.sqrtg * iG1;

@@ -46,17 +46,19 @@ __device__ __forceinline__ T cic_weight(T d)
 // j0+2 is skipped where it does not (its entries are then zero: an end point
 // on theta = pi exactly has b2 = 1).  Element offsets are 32-bit
 // ((n_theta + 1) ld < 2^31).
+template <typename T>
+struct EndWeights {
+    T r0, r1, r2, r3, t0, t1, t2, t3;  // at columns / rows -1 .. 2 of the start cell
+};
+
 template <typename T, int MAXG>
-__device__ __forceinline__ void deposit_warp_split(bool dep, int i0, int j0, int nr, T a1, T a2, T b1, T b2, T cr,
-                                                   T cq, T dphi, int lane, int nth, int ng, int ld, T *J0, T *J1,
-                                                   T *J2)
+__device__ __forceinline__ void deposit_warp(bool dep, int i0, int j0, int nr, T a1, T a2, const EndWeights<T> &S1, int di,
+                                             int dj, T cr, T cq, T dphi, int lane, int nth, int ng, int ld, T *J0, T *J1,
+                                             T *J2)
 {
     const unsigned FULL = 0xffffffffu;
-    // end-point weights at columns / rows -1..2 for b in [-1, 2)
-    const T S1r0 = fmax(T(0), -b1), S1r1 = fmax(T(0), T(1) - fabs(b1)), S1r2 = fmax(T(0), T(1) - fabs(b1 - T(1))),
-            S1r3 = fmax(T(0), b1 - T(1));
-    const T S1t0 = fmax(T(0), -b2), S1t1 = fmax(T(0), T(1) - fabs(b2)), S1t2 = fmax(T(0), T(1) - fabs(b2 - T(1))),
-            S1t3 = fmax(T(0), b2 - T(1));
+    const T S1r0 = S1.r0, S1r1 = S1.r1, S1r2 = S1.r2, S1r3 = S1.r3;
+    const T S1t0 = S1.t0, S1t1 = S1.t1, S1t2 = S1.t2, S1t3 = S1.t3;
     const T S0r1 = T(1) - a1, S0r2 = a1, S0t1 = T(1) - a2, S0t2 = a2;
     const T cp = cq * dphi;
     // prefix sums P(k) = sum_{k' <= k} (S1 - S0)(k'); both weight sets sum to
@@ -71,7 +73,8 @@ __device__ __forceinline__ void deposit_warp_split(bool dep, int i0, int j0, int
     // start-cell group: J^r A (face 1, rows 1, 2), J^th A (columns 1, 2, face
     // 1), J^ph dV (columns 1, 2 x rows 1, 2)
     const T c1 = cr * Pr1, c2 = cr * Pt1;
-    const T core[8] = {c1 * (S1t1 + S0t1), c1 * (S1t2 + S0t2), c2 * (S1r1 + S0r1), c2 * (S1r2 + S0r2),
+    const T St1 = S1t1 + S0t1, St2 = S1t2 + S0t2, Sr1 = S1r1 + S0r1, Sr2 = S1r2 + S0r2;
+    const T core[8] = {c1 * St1, c1 * St2, c2 * Sr1, c2 * Sr2,
                        S1r1 * cU1 + S0r1 * cV1, S1r1 * cU2 + S0r1 * cV2, S1r2 * cU1 + S0r2 * cV1,
                        S1r2 * cU2 + S0r2 * cV2};
     // after the reduction lane (lane & 3) == 0 holds the total of core entry
@@ -126,7 +129,7 @@ __device__ __forceinline__ void deposit_warp_split(bool dep, int i0, int j0, int
         atomicAdd(J2 + (w11 + ld + 1), core[7]);
     }
     // ---- the entries outside the core, lanes that left the start cell
-    const int di = dep ? (int)floor(b1) : 0, dj = dep ? (int)floor(b2) : 0;
+    if (!dep) di = dj = 0;
     if (!__any_sync(FULL, di != 0 || dj != 0)) return;
     // extra column ex = 0 or 3 / face ef = 0 or 2 of an r move, extra row ey
     // = 0 or 3 / theta face eg = 0 or 2 of a theta move, as offsets from the
@@ -136,12 +139,13 @@ __device__ __forceinline__ void deposit_warp_split(bool dep, int i0, int j0, int
     const T Prx = di > 0 ? Pr2 : Pr0, Ptx = dj > 0 ? Pt2 : Pt0;
     const T S1rx = di > 0 ? S1r3 : S1r0, S1tx = dj > 0 ? S1t3 : S1t0;
     const bool row_ok = dj > 0 ? j0 + 2 <= nth : j0 >= 1;  // the extra row exists
+    const T crP = cr * Prx, ctP = cr * Ptx;
     if (di != 0) {
         // J^r A at the extra face, rows 1, 2; J^th A at the extra column,
         // face 1; J^ph at the extra column, rows 1, 2
-        atomicAdd(J0 + (w11 + cf), cr * Prx * (S1t1 + S0t1));
-        atomicAdd(J0 + (w11 + ld + cf), cr * Prx * (S1t2 + S0t2));
-        atomicAdd(J1 + (w11 + cx), cr * S1rx * Pt1);
+        atomicAdd(J0 + (w11 + cf), crP * St1);
+        atomicAdd(J0 + (w11 + ld + cf), crP * St2);
+        atomicAdd(J1 + (w11 + cx), c2 * S1rx);
         atomicAdd(J2 + (w11 + cx), S1rx * cU1);
         atomicAdd(J2 + (w11 + ld + cx), S1rx * cU2);
     }
@@ -149,19 +153,48 @@ __device__ __forceinline__ void deposit_warp_split(bool dep, int i0, int j0, int
         // J^th A at the extra theta face, columns 1, 2; J^r A at face 1, the
         // extra row; J^ph at columns 1, 2, the extra row
         const T u3 = cp3 * S1tx, u6 = cp6 * S1tx;
-        atomicAdd(J1 + (w11 + rg), cr * (S1r1 + S0r1) * Ptx);
-        atomicAdd(J1 + (w11 + rg + 1), cr * (S1r2 + S0r2) * Ptx);
-        atomicAdd(J0 + (w11 + ry), cr * Pr1 * S1tx);
+        atomicAdd(J1 + (w11 + rg), ctP * Sr1);
+        atomicAdd(J1 + (w11 + rg + 1), ctP * Sr2);
+        atomicAdd(J0 + (w11 + ry), c1 * S1tx);
         atomicAdd(J2 + (w11 + ry), S1r1 * u3 + S0r1 * u6);
         atomicAdd(J2 + (w11 + ry + 1), S1r2 * u3 + S0r2 * u6);
+        if (di != 0) {
+            // the corner: J^r A (extra face, extra row), J^th A (extra column,
+            // extra theta face), J^ph (extra column, extra row)
+            atomicAdd(J0 + (w11 + ry + cf), crP * S1tx);
+            atomicAdd(J1 + (w11 + rg + cx), ctP * S1rx);
+            atomicAdd(J2 + (w11 + ry + cx), S1rx * u3);
+        }
     }
-    if (di != 0 && dj != 0 && row_ok) {
-        // the corner: J^r A (extra face, extra row), J^th A (extra column,
-        // extra theta face), J^ph (extra column, extra row)
-        atomicAdd(J0 + (w11 + ry + cf), cr * Prx * S1tx);
-        atomicAdd(J1 + (w11 + rg + cx), cr * S1rx * Ptx);
-        atomicAdd(J2 + (w11 + ry + cx), S1rx * cp3 * S1tx);
-    }
+}
+
+// the deposit for an end point b relative to the start cell (FP32 form)
+template <typename T, int MAXG>
+__device__ __forceinline__ void deposit_warp_split(bool dep, int i0, int j0, int nr, T a1, T a2, T b1, T b2, T cr,
+                                                   T cq, T dphi, int lane, int nth, int ng, int ld, T *J0, T *J1,
+                                                   T *J2)
+{
+    // end-point weights at columns / rows -1..2 for b in [-1, 2)
+    const EndWeights<T> S1 = {fmax(T(0), -b1), fmax(T(0), T(1) - fabs(b1)), fmax(T(0), T(1) - fabs(b1 - T(1))),
+                              fmax(T(0), b1 - T(1)), fmax(T(0), -b2), fmax(T(0), T(1) - fabs(b2)),
+                              fmax(T(0), T(1) - fabs(b2 - T(1))), fmax(T(0), b2 - T(1))};
+    deposit_warp<T, MAXG>(dep, i0, j0, nr, a1, a2, S1, (int)floor(b1), (int)floor(b2), cr, cq, dphi, lane, nth, ng, ld,
+                          J0, J1, J2);
+}
+
+// the deposit for an end point at offsets (f1, f2) in the cell (di, dj) away,
+// di, dj in -1 .. 1 (FP64: the weights by selection, without the comparisons and
+// differences that the FP64 pipe would take)
+template <typename T, int MAXG>
+__device__ __forceinline__ void deposit_warp_cells(bool dep, int i0, int j0, int nr, T a1, T a2, int di, int dj, T f1,
+                                                   T f2, T cr, T cq, T dphi, int lane, int nth, int ng, int ld, T *J0,
+                                                   T *J1, T *J2)
+{
+    const T e1 = T(1) - f1, e2 = T(1) - f2, z = T(0);
+    const EndWeights<T> S1 = {di < 0 ? e1 : z, di < 0 ? f1 : (di == 0 ? e1 : z), di < 0 ? z : (di == 0 ? f1 : e1),
+                              di > 0 ? f1 : z, dj < 0 ? e2 : z, dj < 0 ? f2 : (dj == 0 ? e2 : z),
+                              dj < 0 ? z : (dj == 0 ? f2 : e2), dj > 0 ? f2 : z};
+    deposit_warp<T, MAXG>(dep, i0, j0, nr, a1, a2, S1, di, dj, cr, cq, dphi, lane, nth, ng, ld, J0, J1, J2);
 }
 
 }  // namespace grpic
