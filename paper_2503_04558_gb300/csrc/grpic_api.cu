@@ -414,7 +414,6 @@ grpic_status grpic_init(grpic_metric metric, double spin, const grpic_grid *grid
     if (e == cudaSuccess) e = cudaMalloc(&ctx->d_bigseg, sizeof(int32_t) * (ncell + 1));
     if (e == cudaSuccess) e = cudaMalloc(&ctx->d_offset_prev, sizeof(int32_t) * (ncell + 3));
     if (e == cudaSuccess) e = cudaMalloc(&ctx->d_cnt9, sizeof(int32_t) * 9 * ncell);
-    if (e == cudaSuccess) e = cudaMalloc(&ctx->d_base9, sizeof(int32_t) * 9 * ncell);
     if (e == cudaSuccess) e = cudaMalloc(&ctx->d_sortflag, sizeof(int32_t));
     if (e == cudaSuccess && prm->precision == 64) e = cell_tables(ctx);
     if (e == cudaSuccess) {
@@ -1216,7 +1215,7 @@ void grpic_destroy(grpic_ctx *ctx)
     if (ctx->up_stream) cudaStreamDestroy(ctx->up_stream);
     if (ctx->down_stream) cudaStreamDestroy(ctx->down_stream);
     if (ctx->h_count) cudaFreeHost(ctx->h_count);
-    void *ptrs[] = {ctx->d_spawn, ctx->d_rad, ctx->d_offset_prev, ctx->d_cnt9, ctx->d_base9, ctx->d_sortflag, ctx->rcol, ctx->rcen, ctx->trow, ctx->rcol2, ctx->rowsc, ctx->tab, ctx->col1d, ctx->tab32, ctx->col1d32, ctx->fscratch, ctx->q32, ctx->d_status, ctx->d_keys,
+    void *ptrs[] = {ctx->d_spawn, ctx->d_rad, ctx->d_offset_prev, ctx->d_cnt9, ctx->d_sortflag, ctx->rcol, ctx->rcen, ctx->trow, ctx->rcol2, ctx->rowsc, ctx->tab, ctx->col1d, ctx->tab32, ctx->col1d32, ctx->fscratch, ctx->q32, ctx->d_status, ctx->d_keys,
                     ctx->d_count, ctx->d_offset, ctx->d_cursor, ctx->d_blocksum, ctx->d_perm, ctx->d_bigseg};
     for (void *q : ptrs)
         if (q) cudaFree(q);

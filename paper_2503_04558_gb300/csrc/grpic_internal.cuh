@@ -87,7 +87,6 @@ struct grpic_ctx {
     int32_t *d_bigseg;    // list of oversized segments
     int32_t *d_offset_prev;  // segment offsets of the last sort's output (ncell+3)
     int32_t *d_cnt9;      // per old cell, particles moving in each of 9 directions (9 x ncell)
-    int32_t *d_base9;     // per old cell and direction, the first destination slot (9 x ncell)
     int32_t *d_sortflag;  // 0: neighbour sort applies, 1: general counting sort
     const uint32_t *sorted_tag;  // tag array the last sort wrote
     int64_t pushes_since_sort;

@@ -81,6 +81,7 @@ struct Push32Args {
     int32_t *count;
     int histogram;
     int *status;
+    int runs;  // runs of 256 slots per block
     unsigned long long nr_recip;  // floor(2^64 / n_r) + 1
 };
 
@@ -608,11 +609,9 @@ __device__ __forceinline__ void push_island_df(const Push32Args &A, int i, int j
 
 // PUSHER: 0 generalized Boris, 1 Vay in the FIDO frame; IX: the slot index
 // type (uint32_t while the capacity is below 2^31, int64_t beyond)
-// slots per thread: a block of 256 threads takes GRPIC_PUSH32_PPT consecutive
-// runs of 256 slots in turn (the per-thread setup is paid once for them)
-#ifndef GRPIC_PUSH32_PPT
-#define GRPIC_PUSH32_PPT 8
-#endif
+// slots per thread at most: a block of 256 threads takes consecutive runs of
+// 256 slots in turn
+constexpr int PUSH32_RUNS = 8;
 
 // one slot of the push (all 32 lanes of a warp call it: the deposit and the
 // counts are warp collectives)
@@ -766,10 +765,10 @@ __global__ void __launch_bounds__(256, GRPIC_PUSH32_MINB) push32_kernel(Push32Ar
     int64_t n = permuted ? (int64_t)*A.live : (A.d_count ? *A.d_count : A.n);
     if (n > A.n) n = A.n;
     const IX nx = (IX)n;
-    const IX p0 = (IX)blockIdx.x * (blockDim.x * GRPIC_PUSH32_PPT) + threadIdx.x;
+    const IX p0 = (IX)blockIdx.x * (blockDim.x * (IX)A.runs) + threadIdx.x;
     if (permuted && p0 == 0 && A.count_out) *A.count_out = n;
 #pragma unroll 1
-    for (int k = 0; k < GRPIC_PUSH32_PPT; ++k) push_slot<PUSHER, IX>(A, p0 + (IX)(k * blockDim.x), nx, permuted);
+    for (int k = 0; k < A.runs; ++k) push_slot<PUSHER, IX>(A, p0 + (IX)(k * blockDim.x), nx, permuted);
 }
 
 // The stencil quads of the six field components, interleaved by point (the
@@ -930,8 +929,14 @@ cudaError_t launch_push32(grpic_ctx *ctx, const grpic_particles *in, grpic_parti
     A.status = ctx->d_status;
     A.nr_recip = ~0ull / (unsigned long long)ctx->g.nr + 1ull;
     if (p->n <= 0) return cudaSuccess;
-    const unsigned blocks = (unsigned)((p->n + 256 * GRPIC_PUSH32_PPT - 1) / (256 * GRPIC_PUSH32_PPT));
-    const bool narrow = p->capacity < ((int64_t)1 << 31) - 256 * GRPIC_PUSH32_PPT;
+    // runs of 256 slots per block: PUSH32_RUNS (the per-thread setup paid once for
+    // them), fewer while that would leave under eight rounds of resident blocks
+    // (a last round that is nearly empty, or SMs without work: 2e5 particles in
+    // 98 blocks of 8 runs took 44 us, in 782 of one 19; 2e6: 122 and 99)
+    const int64_t round = (int64_t)256 * GRPIC_PUSH32_MINB * sm_count(ctx->device);
+    A.runs = (int)std::max<int64_t>(1, std::min<int64_t>(PUSH32_RUNS, p->n / (8 * round)));
+    const unsigned blocks = (unsigned)((p->n + 256 * A.runs - 1) / (256 * A.runs));
+    const bool narrow = p->capacity < ((int64_t)1 << 31) - 256 * PUSH32_RUNS;
     if (ctx->prm.pusher) {
         if (narrow)
             push32_kernel<1, uint32_t><<<blocks, 256, 0, s>>>(A);

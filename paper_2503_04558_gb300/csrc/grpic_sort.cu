@@ -392,8 +392,8 @@ struct GatherArgs {
     int64_t nmax;
     const int32_t *live;  // offset[ncell] = number of live particles
     const int32_t *perm;
-    const void *src[6];
-    void *dst[6];
+    const void *src[5];
+    void *dst[5];
     const int32_t *cell_src;
     int32_t *cell_dst;
     const uint32_t *tag_src;
@@ -405,9 +405,8 @@ struct GatherArgs {
 // moves four slots per round (their permutation entries first, then all
 // their loads) so that enough loads are in flight to cover the latency.
 template <typename T>
-__global__ void __launch_bounds__(256) gather_kernel(GatherArgs A, int nfields, const int32_t *flag)
+__global__ void __launch_bounds__(256) gather_kernel(GatherArgs A)
 {
-    if (general_off(flag)) return;
     const int64_t live = *A.live;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     const int64_t s0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -427,7 +426,7 @@ __global__ void __launch_bounds__(256) gather_kernel(GatherArgs A, int nfields, 
             if (src[u] < 0) continue;
 #pragma unroll
             for (int k = 0; k < 5; ++k)
-                if (k < nfields) v[u][k] = ((const T *)A.src[k])[src[u]];
+                v[u][k] = ((const T *)A.src[k])[src[u]];
             tg[u] = A.tag_src[src[u]];
             if (A.cell_dst) cl[u] = A.cell_src[src[u]];
         }
@@ -441,7 +440,7 @@ __global__ void __launch_bounds__(256) gather_kernel(GatherArgs A, int nfields, 
             }
 #pragma unroll
             for (int k = 0; k < 5; ++k)
-                if (k < nfields) ((T *)A.dst[k])[s] = v[u][k];
+                ((T *)A.dst[k])[s] = v[u][k];
             A.tag_dst[s] = tg[u];
             if (A.cell_dst) A.cell_dst[s] = cl[u];
         }
@@ -625,45 +624,97 @@ __global__ void dest_count_kernel(const int32_t *cnt9, int nr, int nth, int32_t 
     }
 }
 
-// first destination slot of old cell s's direction-d particles:
-// offset[k] + arrivals into k from the sources below s in cell order (the
-// directions d' > d), k = s moved by d
-__global__ void base9_kernel(const int32_t *cnt9, int32_t *base9, const int32_t *off_new, int nr, int nth,
-                             const int32_t *flag)
+// Steps 7 when the push itself counted (no fallback can follow): the destination
+// counts and their scan in two launches.  A block sums the arrivals of
+// T * IPT cells and scans them; the second kernel adds the tiles before (at most
+// NSTEP_TILES, read by every block: cheaper than a third launch between them).
+constexpr int NSTEP_TILES = 1024;
+
+template <int T, int IPT>
+__global__ void __launch_bounds__(T) dest_tiles_kernel(const int32_t *cnt9, int nr, int nth, int32_t *out, int32_t *bsum)
 {
-    if (*flag) return;
-    const int64_t ncell = (int64_t)nr * nth;
-    for (int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; s < ncell; s += (int64_t)gridDim.x * blockDim.x) {
-        const int si = (int)(s % nr), sj = (int)(s / nr);
-        int base[9];
+    __shared__ int sh[T / 32];
+    const int64_t ncell = (int64_t)nr * nth, k0 = (int64_t)blockIdx.x * (T * IPT) + threadIdx.x * IPT;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int v[IPT], sum = 0;
+    int ik = (int)(k0 % nr), jk = (int)(k0 / nr);
 #pragma unroll
-        for (int d = 0; d < 9; ++d) {
-            int ik = si + dir_di(d), jk = sj + dir_dj(d);
-            int v = 0;
-            if (ik >= 0 && ik < nr && jk >= 0 && jk < nth) {
-                v = off_new[(int64_t)jk * nr + ik];
+    for (int u = 0; u < IPT; ++u) {
+        int c = 0;
+        if (k0 + u < ncell) {
 #pragma unroll
-                for (int d2 = d + 1; d2 < 9; ++d2) v += arrivals(cnt9, nr, nth, ncell, ik, jk, d2);
-            }
-            base[d] = v;
+            for (int d = 0; d < 9; ++d) c += arrivals(cnt9, nr, nth, ncell, ik, jk, d);
         }
-#pragma unroll
-        for (int d = 0; d < 9; ++d) base9[(int64_t)d * ncell + s] = base[d];
+        v[u] = sum;
+        sum += c;
+        if (++ik == nr) {
+            ik = 0;
+            ++jk;
+        }
     }
+    const int incl = warp_incl_scan(sum);
+    if (lane == 31) sh[warp] = incl;
+    __syncthreads();
+    int base = incl - sum;
+    for (int w = 0; w < warp; ++w) base += sh[w];
+#pragma unroll
+    for (int u = 0; u < IPT; ++u)
+        if (k0 + u <= ncell) out[k0 + u] = v[u] + base;
+    if (threadIdx.x == T - 1) bsum[blockIdx.x] = base + sum;
 }
 
+// out[k] += the tiles before k's; out[n] = the total
+template <int T, int IPT>
+__global__ void __launch_bounds__(T) add_tiles_kernel(int32_t *out, const int32_t *bsum, int64_t n)
+{
+    __shared__ int sh[T / 32];
+    int part = 0;
+    for (int t = threadIdx.x; t < (int)blockIdx.x; t += T) part += bsum[t];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = part;
+    __syncthreads();
+    int base = 0;
+#pragma unroll
+    for (int w = 0; w < T / 32; ++w) base += sh[w];
+    const int64_t k0 = (int64_t)blockIdx.x * (T * IPT);
+#pragma unroll
+    for (int u = 0; u < IPT; ++u) {
+        const int64_t k = k0 + u * T + threadIdx.x;
+        if (k < n) out[k] += base;
+    }
+    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) out[n] = base + bsum[blockIdx.x];
+}
+
+// first destination slot of the direction-d particles of old cell (si, sj):
+// offset[k] + arrivals into k from the sources below it in cell order (the
+// directions d' > d), k the cell moved by d
+__device__ __forceinline__ int first_slot(const int32_t *cnt9, const int32_t *off_new, int nr, int nth, int64_t ncell,
+                                          int si, int sj, int d)
+{
+    const int ik = si + dir_di(d), jk = sj + dir_dj(d);
+    if (ik < 0 || ik >= nr || jk < 0 || jk >= nth) return 0;
+    int v = off_new[(int64_t)jk * nr + ik];
+#pragma unroll
+    for (int d2 = 0; d2 < 9; ++d2)
+        if (d2 > d) v += arrivals(cnt9, nr, nth, ncell, ik, jk, d2);
+    return v;
+}
 
 // step 8: stable placement of the indices: perm[dst] = src, the gather then
 // moves the particle data (one pass with coalesced reads of nearly
 // sequential runs).  A warp streams the keys of TASK_CELLS consecutive old
 // cells; each particle takes the first free slot of its (old cell,
-// direction) run (run counters in shared memory, started at base9), equal
+// direction) run (run counters in shared memory, started at first_slot()), equal
 // (cell, direction) lanes of a chunk taking consecutive slots in lane order.
-__global__ void __launch_bounds__(256) neighbour_perm_kernel(const int32_t *off_old, const int32_t *base9,
-                                                             const int32_t *keys, int nr, int nth, int64_t nmax,
-                                                             int32_t *perm, const int32_t *flag)
+// `per` cells a warp: TASK_CELLS, fewer on small grids so that every SM has work.
+// (first_slot() in a kernel of its own with a table of 9 entries a cell: one more
+// launch, and 72 B a cell written and read.)
+__global__ void __launch_bounds__(256, 8) neighbour_perm_kernel(const int32_t *off_old, const int32_t *off_new,
+                                                             const int32_t *cnt9, const int32_t *keys, int nr, int nth,
+                                                             int per, int64_t nmax, int32_t *perm, const int32_t *flag)
 {
-    if (*flag) return;
+    if (flag && *flag) return;
     __shared__ int run_sh[8][TASK_CELLS * 9];
     const unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
@@ -671,17 +722,24 @@ __global__ void __launch_bounds__(256) neighbour_perm_kernel(const int32_t *off_
     const int64_t ncell = (int64_t)nr * nth;
     const int64_t wid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    const int64_t ntask = (ncell + TASK_CELLS - 1) / TASK_CELLS;
+    const int64_t ntask = (ncell + per - 1) / per;
     for (int64_t t = wid; t < ntask; t += nw) {
-        const int64_t s0 = t * TASK_CELLS;
-        const int m = (int)(ncell - s0 < TASK_CELLS ? ncell - s0 : TASK_CELLS);
+        const int64_t s0 = t * per;
+        const int m = (int)(ncell - s0 < per ? ncell - s0 : per);
         const int o = off_old[s0 + (lane < m ? lane : m)];
         const int end = off_old[s0 + m];
         const int beg = __shfl_sync(FULL, o, 0);
         if (beg >= end) continue;  // warp-uniform
-        if (lane < m)
+        const int s0j = (int)(s0 / nr), s0i = (int)(s0 - (int64_t)s0j * nr);
+        if (lane < m) {
+            int si = s0i + lane, sj = s0j;
+            while (si >= nr) {
+                si -= nr;
+                ++sj;
+            }
 #pragma unroll
-            for (int d = 0; d < 9; ++d) run[lane * 9 + d] = base9[(int64_t)d * ncell + s0 + lane];
+            for (int d = 0; d < 9; ++d) run[lane * 9 + d] = first_slot(cnt9, off_new, nr, nth, ncell, si, sj, d);
+        }
         __syncwarp();
         for (int b = beg; b < end; b += 4 * 32) {
             int kk[4];
@@ -773,6 +831,30 @@ void launch_segfix(grpic_ctx *ctx, int32_t *nbig, const int32_t *flag, cudaStrea
                                                   flag);
 }
 
+// q = p through d_perm (live slots: d_offset[n_cells]), p's count rewritten
+void launch_gather(grpic_ctx *ctx, grpic_particles *p, grpic_particles *q, unsigned blocks, cudaStream_t s)
+{
+    GatherArgs A;
+    A.nmax = p->n;
+    A.live = ctx->d_offset + (int64_t)ctx->g.nr * ctx->g.nth;
+    A.perm = ctx->d_perm;
+    A.tag_src = p->tag;
+    A.tag_dst = q->tag;
+    A.count_out = p->d_count;
+    void *sp[5] = {p->x1, p->x2, p->u1, p->u2, p->u3};
+    void *dp[5] = {q->x1, q->x2, q->u1, q->u2, q->u3};
+    for (int k = 0; k < 5; ++k) {
+        A.src[k] = sp[k];
+        A.dst[k] = dp[k];
+    }
+    A.cell_src = (ctx->prm.precision == 32) ? p->cell : nullptr;
+    A.cell_dst = (ctx->prm.precision == 32) ? q->cell : nullptr;
+    if (ctx->prm.precision == 64)
+        gather_kernel<double><<<blocks, 256, 0, s>>>(A);
+    else
+        gather_kernel<float><<<blocks, 256, 0, s>>>(A);
+}
+
 }  // namespace
 
 // Expects ctx->d_keys / ctx->d_count filled for the current order of *p.
@@ -798,31 +880,7 @@ cudaError_t launch_sort(grpic_ctx *ctx, grpic_particles *p, grpic_particles *q, 
     // so a fixed grid strides over it and returns at once when it is empty
     bigseg_kernel<<<64, 1024, SEG_BLOCK_MAX * sizeof(int), s>>>(ctx->d_offset, ctx->d_perm, ctx->d_bigseg, nbig,
                                                                 nullptr);
-    GatherArgs A;
-    A.nmax = p->n;
-    A.live = ctx->d_offset + ncell;
-    A.perm = ctx->d_perm;
-    A.tag_src = p->tag;
-    A.tag_dst = q->tag;
-    A.count_out = p->d_count;
-    int nf = 5;
-    void *sp[5] = {p->x1, p->x2, p->u1, p->u2, p->u3};
-    void *dp[5] = {q->x1, q->x2, q->u1, q->u2, q->u3};
-    for (int k = 0; k < 5; ++k) {
-        A.src[k] = sp[k];
-        A.dst[k] = dp[k];
-    }
-    A.src[5] = nullptr;
-    A.dst[5] = nullptr;
-    A.cell_src = (ctx->prm.precision == 32) ? p->cell : nullptr;
-    A.cell_dst = (ctx->prm.precision == 32) ? q->cell : nullptr;
-    if (p->n > 0) {
-        unsigned blocks = (unsigned)((p->n + 255) / 256);
-        if (ctx->prm.precision == 64)
-            gather_kernel<double><<<blocks, 256, 0, s>>>(A, nf, nullptr);
-        else
-            gather_kernel<float><<<blocks, 256, 0, s>>>(A, nf, nullptr);
-    }
+    if (p->n > 0) launch_gather(ctx, p, q, (unsigned)((p->n + 255) / 256), s);
     return cudaGetLastError();
 }
 
@@ -846,17 +904,39 @@ cudaError_t launch_sort_step(grpic_ctx *ctx, grpic_particles *p, grpic_particles
     const int ncell = ctx->g.nr * ctx->g.nth;
     const int64_t nscan = (int64_t)ncell + 1;
     const int nb = (int)((nscan + SCAN_TILE - 1) / SCAN_TILE);
-    int dev_sms = 152;
-    cudaDeviceGetAttribute(&dev_sms, cudaDevAttrMultiProcessorCount, ctx->device);
+    const int dev_sms = sm_count(ctx->device);
     const unsigned grid = (unsigned)dev_sms * 8;  // fixed grids, strided work
+    const int64_t gmax = (int64_t)dev_sms * 64;
+    const unsigned gp = (unsigned)std::max<int64_t>(1, std::min<int64_t>((p->n + 255) / 256, gmax));
     int32_t *flag = ctx->d_sortflag;
-    if (neighbour && ctx->g.nr >= 3) {
+    int per = TASK_CELLS;
+    while (per > 4 && ncell < (int64_t)per * grid * 8) per >>= 1;
+    if (neighbour && counts_ready) {
+        // The push that read through the last sort's permutation counted: its
+        // slots are that sort's segments and its moves at most one cell, by
+        // construction, so no fallback is launched (7 launches that would find
+        // nothing to do; at 128^2 the sort goes from 56 to 16 us of the step).
+        if (nscan <= (int64_t)NSTEP_TILES * 1024) {
+            const unsigned tiles = (unsigned)((nscan + 1023) / 1024);
+            dest_tiles_kernel<256, 4><<<tiles, 256, 0, s>>>(ctx->d_cnt9, ctx->g.nr, ctx->g.nth, ctx->d_offset,
+                                                            ctx->d_blocksum);
+            add_tiles_kernel<256, 4><<<tiles, 256, 0, s>>>(ctx->d_offset, ctx->d_blocksum, nscan);
+        } else {
+            dest_tiles_kernel<SCAN_T, SCAN_IPT><<<nb, SCAN_T, 0, s>>>(ctx->d_cnt9, ctx->g.nr, ctx->g.nth, ctx->d_offset,
+                                                                      ctx->d_blocksum);
+            scan_sums<<<1, SCAN_T, 0, s>>>(ctx->d_blocksum, nb, ctx->d_offset + nscan);
+            add_back<<<(unsigned)((nscan + 255) / 256), 256, 0, s>>>(ctx->d_offset, ctx->d_blocksum, nscan);
+        }
+        if (p->n > 0)
+            neighbour_perm_kernel<<<grid, 256, 0, s>>>(ctx->d_offset_prev, ctx->d_offset, ctx->d_cnt9, ctx->d_keys,
+                                                       ctx->g.nr, ctx->g.nth, per, p->n, ctx->d_perm, nullptr);
+        if (p->n > 0 && materialize) launch_gather(ctx, p, q, gp, s);
+        return cudaGetLastError();
+    }
+    if (neighbour) {
         cudaMemsetAsync(flag, 0, sizeof(int32_t), s);
-        // (a push that read through the last sort's permutation counted
-        // already: its slots are that sort's segments by construction)
-        if (!counts_ready)
-            count9_kernel<<<grid, 256, 0, s>>>(ctx->d_offset_prev, ctx->d_keys, ctx->g.nr, ncell, p->d_count, p->n,
-                                               ctx->d_cnt9, flag);
+        count9_kernel<<<grid, 256, 0, s>>>(ctx->d_offset_prev, ctx->d_keys, ctx->g.nr, ncell, p->d_count, p->n,
+                                           ctx->d_cnt9, flag);
         dest_count_kernel<<<grid, 256, 0, s>>>(ctx->d_cnt9, ctx->g.nr, ctx->g.nth, ctx->d_count, flag);
         if (hist_on_fallback) {
             // the push skipped the histogram: rebuild it if the device fell back
@@ -871,49 +951,22 @@ cudaError_t launch_sort_step(grpic_ctx *ctx, grpic_particles *p, grpic_particles
     scan_tiles<<<nb, SCAN_T, 0, s>>>(ctx->d_count, ctx->d_offset, ctx->d_blocksum, nscan);
     scan_sums<<<1, SCAN_T, 0, s>>>(ctx->d_blocksum, nb, ctx->d_offset + nscan);
     add_back<<<(unsigned)((nscan + 255) / 256), 256, 0, s>>>(ctx->d_offset, ctx->d_blocksum, nscan);
-    if (neighbour && ctx->g.nr >= 3 && p->n > 0) {
-        base9_kernel<<<grid, 256, 0, s>>>(ctx->d_cnt9, ctx->d_base9, ctx->d_offset, ctx->g.nr, ctx->g.nth, flag);
-        neighbour_perm_kernel<<<grid, 256, 0, s>>>(ctx->d_offset_prev, ctx->d_base9, ctx->d_keys, ctx->g.nr,
-                                                   ctx->g.nth, p->n, ctx->d_perm, flag);
-    }
+    if (neighbour && p->n > 0)
+        neighbour_perm_kernel<<<grid, 256, 0, s>>>(ctx->d_offset_prev, ctx->d_offset, ctx->d_cnt9, ctx->d_keys,
+                                                   ctx->g.nr, ctx->g.nth, per, p->n, ctx->d_perm, flag);
     // general path to the permutation (skipped on the device when the neighbour sort applied)
-    cudaMemsetAsync(ctx->d_cursor, 0, sizeof(int32_t) * nscan, s);
     int32_t *nbig = ctx->d_cursor + nscan;
-    cudaMemsetAsync(nbig, 0, sizeof(int32_t), s);
+    cudaMemsetAsync(ctx->d_cursor, 0, sizeof(int32_t) * (nscan + 1), s);  // with the count behind the cursors
     // general path grids: enough blocks for memory parallelism, few enough
     // that skipping them costs little
-    const int64_t gmax = (int64_t)dev_sms * 64;
-    const unsigned gp = (unsigned)std::max<int64_t>(1, std::min<int64_t>((p->n + 255) / 256, gmax));
     if (p->n > 0)
         scatter_kernel<<<gp, 256, 0, s>>>(p->n, p->d_count, ctx->d_keys, ctx->d_offset, ctx->d_cursor, ctx->d_perm,
                                           ncell, flag);
     launch_segfix(ctx, nbig, flag, s);
     bigseg_kernel<<<64, 1024, SEG_BLOCK_MAX * sizeof(int), s>>>(ctx->d_offset, ctx->d_perm, ctx->d_bigseg, nbig, flag);
-    GatherArgs G;
-    G.nmax = p->n;
-    G.live = ctx->d_offset + ncell;
-    G.perm = ctx->d_perm;
-    G.tag_src = p->tag;
-    G.tag_dst = q->tag;
-    G.count_out = p->d_count;
-    void *sp[5] = {p->x1, p->x2, p->u1, p->u2, p->u3};
-    void *dp[5] = {q->x1, q->x2, q->u1, q->u2, q->u3};
-    for (int k = 0; k < 5; ++k) {
-        G.src[k] = sp[k];
-        G.dst[k] = dp[k];
-    }
-    G.src[5] = nullptr;
-    G.dst[5] = nullptr;
-    G.cell_src = (ctx->prm.precision == 32) ? p->cell : nullptr;
-    G.cell_dst = (ctx->prm.precision == 32) ? q->cell : nullptr;
     // both paths leave the permutation in d_perm: one gather moves the data
     // (or the next push reads through it)
-    if (p->n > 0 && materialize) {
-        if (ctx->prm.precision == 64)
-            gather_kernel<double><<<gp, 256, 0, s>>>(G, 5, nullptr);
-        else
-            gather_kernel<float><<<gp, 256, 0, s>>>(G, 5, nullptr);
-    }
+    if (p->n > 0 && materialize) launch_gather(ctx, p, q, gp, s);
     return cudaGetLastError();
 }
 
