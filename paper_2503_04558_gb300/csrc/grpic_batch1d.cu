@@ -20,6 +20,12 @@
 // identical copies of D^r, the second CTA's survivors are moved down behind
 // the first's and the children follow in parent order: the same line state
 // as one CTA would leave, up to the rounding of the current's sum.
+//
+// Bound by instruction issue (70 % of the slots, about 910 instructions per
+// particle-step before any photon).  20 steps of 512 lines x 4096 cells, 1.03e7
+// particles: 10.26 -> 9.41 ms with the currents' sums in 32-bit words, divisions
+// by tabulated values through their inverses (the same results bit for bit), the
+// ranks by ballots and the emission's FP32 screen on hardware reciprocals.
 #include "grpic_geo.cuh"
 #include "grpic_philox.cuh"
 
@@ -44,7 +50,9 @@ struct B1Args {
     // per-particle work kept off the FP64 pipe: r_i in FP32, the FP32 screen of
     // the emission threshold, the conversion probability as a 53-bit integer
     // threshold (bits < ceil(P 2^53) exactly when the uniform is below P)
-    const float *rcolf;
+    const float *rcolf, *ircolf;  // r_i and 1 / r_i
+    float idx1f;                  // 1 / dx1f
+    float cq[4];                  // -q w / dt per species
     float gthr2s;
     uint64_t pconv53;
     int n_iter;
@@ -102,20 +110,49 @@ __device__ __forceinline__ float W1f(float d)
     return d < 1.0f ? 1.0f - d : 0.0f;
 }
 
-// block-wide exclusive scan of one int per thread; returns the total.  No
+// a / b, correctly rounded, from inv = 1 / b correctly rounded (Markstein): three
+// operations for the FP32 division's eight and its branch
+__device__ __forceinline__ float div_by(float a, float b, float inv)
+{
+    const float q = a * inv;
+    return fmaf(fmaf(-q, b, a), inv, q);
+}
+
+// v added to the 64-bit sum held as two 32-bit words: the low word's carry goes
+// into the high one, which most contributions then leave alone.  (The shared
+// memory has no 64-bit add: as a compare-and-swap loop it measured 1.7 a clock and
+// SM, two 32-bit adds 6.0.)
+__device__ __forceinline__ void add64(uint32_t *lo, uint32_t *hi, int at, long long v)
+{
+    const uint32_t l = (uint32_t)v;
+    const uint32_t old = atomicAdd(lo + at, l);
+    const uint32_t h = (uint32_t)((unsigned long long)v >> 32) + (old + l < l ? 1u : 0u);
+    if (h) atomicAdd(hi + at, h);
+}
+__device__ __forceinline__ long long sum64(const uint32_t *lo, const uint32_t *hi, int at)
+{
+    return (long long)(((unsigned long long)hi[at] << 32) | lo[at]);
+}
+
+// block-wide exclusive ranks of this thread's survivor and of its children among
+// all threads' (excl: survivors in the low half, children in the high half) and
+// their totals, packed alike; the per-thread values are a bit and 0, 1 or 2, so a
+// warp ranks them by ballots.  No
 // barrier after the totals are read: successive calls alternate between two
 // wsum buffers (a warp can start the call after next only once every thread
 // has passed the next call's first barrier, so this call's buffer is free)
-__device__ __forceinline__ int block_scan(int v, int *wsum, int &excl)
+__device__ __forceinline__ int block_ranks(bool alive, int napp, int *wsum, int &excl)
 {
-    int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
-    int x = v;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        int y = __shfl_up_sync(0xffffffffu, x, o);
-        if (lane >= o) x += y;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
+    const unsigned below = (1u << lane) - 1u;
+    const unsigned ma = __ballot_sync(0xffffffffu, alive);
+    int own = __popc(ma & below), x = __popc(ma);
+    if (__any_sync(0xffffffffu, napp != 0)) {
+        const unsigned m1 = __ballot_sync(0xffffffffu, napp & 1), m2 = __ballot_sync(0xffffffffu, napp & 2);
+        own |= (__popc(m1 & below) + 2 * __popc(m2 & below)) << 16;
+        x |= (__popc(m1) + 2 * __popc(m2)) << 16;
     }
-    if (lane == 31) wsum[warp] = x;
+    if (lane == 0) wsum[warp] = x;
     __syncthreads();
     if (warp == 0) {
         int w = lane < nw ? wsum[lane] : 0;
@@ -129,7 +166,7 @@ __device__ __forceinline__ int block_scan(int v, int *wsum, int &excl)
         if (lane == 31) wsum[32] = wi;
     }
     __syncthreads();
-    excl = wsum[warp] + x - v;
+    excl = wsum[warp] + own;
     return wsum[32];
 }
 
@@ -150,8 +187,8 @@ __device__ __forceinline__ void b1_body(const B1Args &A)
     // J^r A_r at faces -1..n in fixed point (units of A.junit): integer sums
     // do not depend on the order of the atomics, so a line's current is the
     // same whichever warps and CTAs deposit it
-    long long *sJ = reinterpret_cast<long long *>(smem);
-    float *sD = reinterpret_cast<float *>(sJ + n + 2);
+    uint32_t *sJlo = reinterpret_cast<uint32_t *>(smem), *sJhi = sJlo + n + 2;
+    float *sD = reinterpret_cast<float *>(sJhi + n + 2);
     float *sA = sD + n;
     int *wsum = (int *)(sA + n);             // two scan buffers of 33 ints (34 apart)
     int *sv = wsum + 68;                     // [0] line, [3] emitted, [4] converted, [5] pushed,
@@ -179,6 +216,7 @@ __device__ __forceinline__ void b1_body(const B1Args &A)
         double sd, cd;
         sincos(th, &sd, &cd);
         const float sf = (float)sd, cf = (float)cd;
+        const float is2f = 1.0f / (sf * sf);
         const float I0 = (float)A.I0[k];
         for (int i = tid; i < n; i += B) {
             sD[i] = A.D[(size_t)k * n + i];
@@ -191,7 +229,7 @@ __device__ __forceinline__ void b1_body(const B1Args &A)
         for (int st = 0; st < A.nsteps; ++st) {
             const int64_t step = A.step0 + st;
             const int src = (A.cur + st) & 1, dst = src ^ 1;
-            for (int i = tid; i < n + 2; i += B) sJ[i] = 0;
+            for (int i = tid; i < 2 * (n + 2); i += B) sJlo[i] = 0;
             if (tid == 0) {
                 sv[3] = 0;
                 sv[4] = 0;
@@ -256,7 +294,7 @@ __device__ __forceinline__ void b1_body(const B1Args &A)
                         dl = d0 + h * (ft.xr + f0.xr);
                         u1 = ur + h * (ft.ur + f0.ur);
                     }
-                    float on = log1pf(dl / rcf) / A.dx1f;
+                    float on = div_by(log1pf(div_by(dl, rcf, A.ircolf[ci])), A.dx1f, A.idx1f);
                     if (!(isfinite(on) && isfinite(u1) && rcf + dl > 0.0f)) {
                         set_status(A.status, GRPIC_ENAN);
                     } else {
@@ -266,14 +304,16 @@ __device__ __forceinline__ void b1_body(const B1Args &A)
                         } else {
                             if (A.qw[sp] != 0.0f) {
                                 // 1D Esirkepov: J A(face f) -= (q/dt) sum_{k'<=f} (S1 - S0)
-                                float acc = 0.0f, cq = -A.qw[sp] / A.dtf;
+                                // (the start offset o in [0, 1) has no weight at
+                                // nodes -1 and 2)
+                                float acc = 0.0f;
+                                const float cq = A.cq[sp];
 #pragma unroll
                                 for (int w = 0; w < 4; ++w) {
-                                    acc += W1f(on - (float)(w - 1)) - W1f(o - (float)(w - 1));
+                                    acc += W1f(on - (float)(w - 1)) - (w == 1 || w == 2 ? W1f(o - (float)(w - 1)) : 0.0f);
                                     int face = ci - 1 + w;
                                     if (acc != 0.0f && face >= -1 && face <= n)
-                                        atomicAdd(reinterpret_cast<unsigned long long *>(&sJ[face + 1]),
-                                                  (unsigned long long)fixed_units(cq * acc * A.jinv));
+                                        add64(sJlo, sJhi, face + 1, fixed_units(cq * acc * A.jinv));
                                 }
                             }
                             int ni = ci + di;
@@ -288,10 +328,13 @@ __device__ __forceinline__ void b1_body(const B1Args &A)
                                 // FP64 decisions at the new position
                                 if (massive && charged) {
                                     // FP32 screen, FP64 decision inside the ambiguity band
-                                    float rf = A.rcolf[ci] * (1.0f + expm1f(o * A.dx1f));
-                                    float rho2 = rf * rf + A.af * A.af * cf * cf, ir = 1.0f / rho2, z = 2.0f * rf * ir;
-                                    float gr = (A.af * A.af + rf * rf) * ir - z / (1.0f + z), gp = A.af * ir,
-                                          gq = ir / (sf * sf);
+                                    // (r = r_i + dl of the push; hardware reciprocals:
+                                    // the band is 1e-4 wide)
+                                    const float rf = rcf + dl;
+                                    const float rho2 = fmaf(rf, rf, A.af * A.af * cf * cf), ir = rcp_t(rho2),
+                                                z = 2.0f * rf * ir;
+                                    const float gr = (A.af * A.af + rf * rf) * ir - z * rcp_t(1.0f + z), gp = A.af * ir,
+                                                gq = ir * is2f;
                                     float G2 = 1.0f + gr * ur * ur + 2.0f * gp * ur * up + gq * up * up;
                                     if (G2 >= A.gthr2s) {
                                         double rd = A.rcol[ci] * exp((double)o * A.dx1), grr, grp, gpp;
@@ -343,7 +386,7 @@ __device__ __forceinline__ void b1_body(const B1Args &A)
                 }
                 // placement: survivors in order, children in parent order
                 int excl;
-                int tot = block_scan((alive ? 1 : 0) | (napp << 16), wsum + (((cb - lo) / B) & 1) * 34, excl);
+                int tot = block_ranks(alive, napp, wsum + (((cb - lo) / B) & 1) * 34, excl);
                 if (alive) {
                     size_t d = base + lo + wp + (excl & 0xffff);
                     A.cell[dst][d] = ci;
@@ -389,9 +432,9 @@ __device__ __forceinline__ void b1_body(const B1Args &A)
                 }
                 cnt = wptr + ncopy;
                 // field: d(A D)/dt = I0 - J A
-                for (int i = tid; i < n; i += B) sD[i] += A.dtf * (I0 - __ll2float_rn(sJ[i + 1]) * A.junit) / sA[i];
+                for (int i = tid; i < n; i += B) sD[i] += A.dtf * (I0 - __ll2float_rn(sum64(sJlo, sJhi, i + 1)) * A.junit) / sA[i];
                 if (A.JA && st == A.nsteps - 1)
-                    for (int i = tid; i < n + 2; i += B) A.JA[(size_t)k * (n + 2) + i] = __ll2float_rn(sJ[i]) * A.junit;
+                    for (int i = tid; i < n + 2; i += B) A.JA[(size_t)k * (n + 2) + i] = __ll2float_rn(sum64(sJlo, sJhi, i)) * A.junit;
             } else {
                 cg::cluster_group cl = cg::this_cluster();
                 if (tid == 0) {
@@ -404,12 +447,13 @@ __device__ __forceinline__ void b1_body(const B1Args &A)
                 const int K0 = (int)min((int64_t)v0[7], CsR), K1 = (int)min((int64_t)v1[7], CsR);
                 // field with the current of the whole line, summed in rank order so
                 // that both copies of D^r stay identical
-                const long long *J0 = cl.map_shared_rank(sJ, 0), *J1 = cl.map_shared_rank(sJ, 1);
-                for (int i = tid; i < n; i += B)
-                    sD[i] += A.dtf * (I0 - __ll2float_rn(J0[i + 1] + J1[i + 1]) * A.junit) / sA[i];
+                const uint32_t *l0 = cl.map_shared_rank(sJlo, 0), *l1 = cl.map_shared_rank(sJlo, 1);
+                const uint32_t *h0 = l0 + (n + 2), *h1 = l1 + (n + 2);
+                auto line_j = [&](int i) { return __ll2float_rn(sum64(l0, h0, i) + sum64(l1, h1, i)) * A.junit; };
+                for (int i = tid; i < n; i += B) sD[i] += A.dtf * (I0 - line_j(i + 1)) / sA[i];
                 if (A.JA && st == A.nsteps - 1 && rank == 0)
                     for (int i = tid; i < n + 2; i += B)
-                        A.JA[(size_t)k * (n + 2) + i] = __ll2float_rn(J0[i] + J1[i]) * A.junit;
+                        A.JA[(size_t)k * (n + 2) + i] = line_j(i);
                 // rank 1's survivors (written from its first particle's slot) move
                 // down behind rank 0's, a chunk at a time: every chunk is read
                 // before it is written and its destination lies below the next
@@ -595,6 +639,9 @@ B1Args make_args(grpic_batch1d_ctx *c, grpic_lines *L, int nsteps, int64_t step0
     A.junit = (float)unit;
     A.jinv = (float)(1.0 / unit);
     A.rcolf = c->rcolf;
+    A.ircolf = c->rcolf + (p.n_cells + 1);
+    A.idx1f = 1.0f / A.dx1f;
+    for (int s = 0; s < 4; ++s) A.cq[s] = -A.qw[s] / A.dtf;
     A.gthr2s = (float)(p.gamma_thr * p.gamma_thr) * 0.9999f;
     A.pconv53 = (uint64_t)std::ceil(A.Pconv * 9007199254740992.0);
     A.theta = L->theta;
@@ -706,7 +753,7 @@ grpic_status grpic_batch1d_init(const grpic_batch1d_params *p, grpic_batch1d_ctx
     c->smem = sizeof(long long) * ((size_t)n + 2) + sizeof(float) * 2 * (size_t)n + sizeof(int) * 80;
     size_t ns = (size_t)p->n_lines * c->Cs;
     cudaError_t e = cudaMalloc(&c->rcol, sizeof(double) * (n + 1));
-    if (e == cudaSuccess) e = cudaMalloc(&c->rcolf, sizeof(float) * (n + 1));
+    if (e == cudaSuccess) e = cudaMalloc(&c->rcolf, sizeof(float) * 2 * (n + 1));
     if (e == cudaSuccess) e = cudaMalloc(&c->Ar, sizeof(float) * (size_t)p->n_lines * n);
     if (e == cudaSuccess) e = cudaMalloc(&c->order, sizeof(int32_t) * p->n_lines);
     if (e == cudaSuccess) e = cudaMalloc(&c->queue, sizeof(int32_t) * 4);
@@ -729,7 +776,8 @@ grpic_status grpic_batch1d_init(const grpic_batch1d_params *p, grpic_batch1d_ctx
     for (int i = 0; i <= n; ++i) r[i] = p->r_in * std::exp(i * dx1);
     cudaMemcpy(c->rcol, r.data(), sizeof(double) * (n + 1), cudaMemcpyHostToDevice);
     std::vector<float> rf(r.begin(), r.end());
-    cudaMemcpy(c->rcolf, rf.data(), sizeof(float) * (n + 1), cudaMemcpyHostToDevice);
+    for (int i = 0; i <= n; ++i) rf.push_back(1.0f / rf[i]);  // the inverses behind
+    cudaMemcpy(c->rcolf, rf.data(), sizeof(float) * 2 * (n + 1), cudaMemcpyHostToDevice);
     cudaMemset(c->status, 0, sizeof(int) * 4);
     // default launch shape until the tuner picks one
     c->block = 256;
