@@ -96,6 +96,16 @@ __device__ __forceinline__ df sqrt_t(const df &x)
     return fast_two_sum(s0, __fmul_rn(e, __fmul_rn(0.5f, y0)));
 }
 
+// 1/sqrt(x): y0 ~ 1/sqrt(x.hi) (2 ulp) and one Newton step with the residual
+// 1 - x y0^2 in FP32 from the exact product y0^2 (its rounding stays below 2^-45)
+__device__ __forceinline__ df rsqrt_t(const df &x)
+{
+    const float y0 = rsqrtf(x.hi);
+    const df q = two_prod(y0, y0);
+    const float e = fmaf(-x.lo, q.hi, fmaf(-x.hi, q.lo, fmaf(-x.hi, q.hi, 1.0f)));
+    return fast_two_sum(y0, __fmul_rn(__fmul_rn(0.5f, y0), e));
+}
+
 // 2^k x: exact scaling of both parts
 __device__ __forceinline__ df scale2(const df &x, float p2) { return df(__fmul_rn(x.hi, p2), __fmul_rn(x.lo, p2)); }
 
@@ -139,5 +149,27 @@ __device__ __forceinline__ void sincos_shift_df(const df &s0, const df &c0, cons
     s = add_f(s0 + c0 * d, -fmaf(s0.hi, ec, c0.hi * xes));
     c = add_f(c0 - s0 * d, -fmaf(c0.hi, ec, -s0.hi * xes));
 }
+
+// ---------------------------------------------------------------------------
+// Between pairs and doubles by integer operations (the FP64 pipe takes each
+// conversion at the price of a multiply-add): a double's leading 24 significant
+// bits and the 24 after them; magnitudes below 2^-74 become 0
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ df df_of(double x)
+{
+    const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+    const unsigned sign = hi & 0x80000000u;
+    const int e = (int)((hi >> 20) & 0x7ffu);
+    const float h = __uint_as_float(((__funnelshift_l(lo, hi, 3) - 0xC0000000u) & 0x7fffffffu) | sign);
+    const float ulp = __uint_as_float(((unsigned)(e - 1075 + 127) << 23) | sign);  // 2^(e - 1075), x's last bit
+    if (e < 950) return df(0.0f);
+    return fast_two_sum(h, __fmul_rn(__int2float_rn((int)(lo & 0x1fffffffu)), ulp));
+}
+__device__ __forceinline__ double double_of_float(float x)
+{
+    const unsigned u = __float_as_uint(x);
+    return __hiloint2double((int)((((u & 0x7fffffffu) >> 3) + 0x38000000u) | (u & 0x80000000u)), (int)(u << 29));
+}
+__device__ __forceinline__ double double_of(const df &x) { return double_of_float(x.hi) + double_of_float(x.lo); }
 
 }  // namespace grpic

@@ -23,10 +23,13 @@
 // and a short series, sin and cos from the row's, reciprocals and roots from
 // hardware seeds and one third-order step, sign and range tests and selections
 // from the bits.  1.68e7 particles on 512^2: 25.7 -> 17.5 ms (766 -> about 530 pipe
-// instructions a particle); the errors against 64 bits are no larger (u_theta
-// near the axis a third to a half of before, J^r 1.3e-12 -> 0.9e-12).
+// instructions a particle), and 12.0 ms with the early correctors in double-FP32
+// pairs; the errors against 64 bits are no larger (positions 1.9e-18 before and
+// after, J^r 1.3e-12 -> 0.9e-12, u_theta, set by the few particles at the axis,
+// within the seeds' spread, and the same with and without the pairs).
 #include "grpic_internal.cuh"
 #include "grpic_geo.cuh"
+#include "grpic_df.cuh"
 #include "grpic_window.cuh"
 #include "grpic_vay.cuh"
 #include "grpic_shape3.cuh"
@@ -40,6 +43,9 @@ struct Push64Args {
     double dt;
     double idt, m_i2dt;  // 1 / dt, -1 / (2 dt)
     int n_iter;
+    int pairs;           // the correctors before the last may run in pairs
+    float hf;            // dt / 2
+    df a_df, a2_df, dt_df;
     double qm[4], qw[4];
     double qdt[4], wr[4], wp[4];  // q dt / (2 m); -q w / (2 dt), q w / dt
     int massive[4];
@@ -94,6 +100,98 @@ __device__ __forceinline__ void geo_rhs_sc(double a, double a2, double m2a2, dou
 {
     const Pt64 m = pointT<double>(a2, m2a2, r, s, c);
     rhsT<double>(m, a, eps, ur, ut, up, a * up, f);
+}
+
+// The correctors before the last one in double-FP32 pairs (about 44 significant
+// bits on the FP32 pipes, which the push leaves idle).  Their result is only
+// the point where the last corrector, in FP64, takes its right-hand side: an error
+// eps of an iterate comes out of it times (dt/2 dF/dy)^2, of the order of the
+// square of dt/2 times the angular velocity or the inverse radius.  They run
+// where that square is below 2^-14 (PAIR_MAX_ANGLE, PAIR_MAX_DT; eps times it is
+// then under an eighth of an FP64 rounding), and in FP64 elsewhere: next to
+// the axis and on coarse grids.  Per particle, so that a result does not depend
+// on the warp's other lanes.
+constexpr float PAIR_MAX_ANGLE = 0.0064f;  // of dt/2 |dphi/dt|
+constexpr double PAIR_MAX_DT = 0.02;
+
+struct RhsDf {
+    df xr, xt, ur, ut;
+};
+
+// rhsT's right-hand side (without X^phi) in pairs at (r, sin, cos theta, u)
+__device__ __forceinline__ void geo_rhs_df(const df &a2, float eps, const df &r, const df &s, const df &c, const df &ur,
+                                           const df &ut, const df &up, const df &aup, RhsDf &f)
+{
+    const df r2 = r * r;
+    const df ir = rcp_t(r2 + a2 * (c * c));
+    const df z = scale2(r, 2.0f) * ir;
+    const df opz = add_f(z, 1.0f);
+    const df iopz = rcp_t(opz);
+    const df beta = z * iopz;
+    const df is2 = rcp_t(s * s);
+    const df ar2 = a2 + r2;
+    const df cs = c * s;
+    const df E = scale2(a2 * cs, -2.0f) * ir;
+    const df ur2 = ur * ur;
+    const df is2up2 = is2 * up * up;
+    const df w = ar2 * ur + aup;
+    const df P = ur * (w + aup) + (ut * ut + is2up2);
+    const df irP = ir * P;
+    const df Q = add_f(irP - beta * ur2, eps);
+    const df iu0 = rsqrt_t(opz * Q);
+    const df h = scale2(iu0, 0.5f);
+    const df iri = ir * iu0;
+    f.xr = iu0 * (ir * w - beta * ur) - beta;
+    f.xt = iri * ut;
+    const df K = iopz * (iopz * ur * add_f(h * ur, 1.0f) + h * Q);
+    f.ur = K * (scale2(ir, 2.0f) - z * z) + h * z * (irP - ur2);
+    f.ut = E * (h * irP - K * z) + iri * (cs * is2) * is2up2;
+}
+
+// sin, cos of (theta0 + d), |d| <= 0.03: the second-order terms in pairs, the
+// rest of the series (d^4 / 24) in FP32
+__device__ __forceinline__ void sincos_shift_pair(const df &s0, const df &c0, const df &d, df &s, df &c)
+{
+    const df d2 = d * d;
+    const float q = __fmul_rn(d2.hi, d2.hi);
+    const df ec = add_f(scale2(d2, 0.5f), -q * fmaf(d2.hi, -1.0f / 720.0f, 1.0f / 24.0f));  // 1 - cos d
+    const df es = add_f(d2 * df_const(1.0 / 6.0), -q * (1.0f / 120.0f));                    // 1 - sin(d) / d
+    const df cd = c0 * d, sd = s0 * d;
+    s = (s0 + cd) - (s0 * ec + cd * es);
+    c = (c0 - sd) - (c0 * ec - sd * es);
+}
+
+// n correctors in pairs from the predictor: on return the changes of r, theta,
+// u_r, u_theta against x^n; false (nothing kept) where an iterate leaves the range
+__device__ __forceinline__ bool correctors_df(const df &a, const df &a2, const df &dt, int n, float eps, double r,
+                                              double s0, double c0, const double u[3], const Rhs &f0, double &dr,
+                                              double &dth, double &dur, double &dut)
+{
+    const df R = df_of(r), S0 = df_of(s0), C0 = df_of(c0), U0 = df_of(u[0]), U1 = df_of(u[1]), up = df_of(u[2]);
+    const df aup = a * up, h = scale2(dt, 0.5f);
+    const df x0 = df_of(f0.xr), t0 = df_of(f0.xt), v0 = df_of(f0.ur), w0 = df_of(f0.ut);
+    df dR = dt * x0, dT = dt * t0, dV = dt * v0, dW = dt * w0;
+    // theta may move by a few hundredths, and by an eighth of its distance to the
+    // axis (the angular velocity of the criterion is that of x^n)
+    const float room = fminf(4.0f * PAIR_MAX_ANGLE, 0.125f * S0.hi);
+#pragma unroll 1
+    for (int it = 0; it < n; ++it) {
+        if (!(fabsf(dT.hi) < room)) return false;
+        df s, c;
+        sincos_shift_pair(S0, C0, dT, s, c);
+        RhsDf f;
+        geo_rhs_df(a2, eps, R + dR, s, c, U0 + dV, U1 + dW, up, aup, f);
+        dR = h * (f.xr + x0);
+        dT = h * (f.xt + t0);
+        dV = h * (f.ur + v0);
+        dW = h * (f.ut + w0);
+    }
+    if (!(fabsf(dT.hi) < room)) return false;
+    dr = double_of(dR);
+    dth = double_of(dT);
+    dur = double_of(dV);
+    dut = double_of(dW);
+    return true;
 }
 
 // the 3+1 metric at the point (App. A): gamma_rr = 1 + z, gamma_thth = rho^2,
@@ -311,10 +409,23 @@ __global__ void __launch_bounds__(256) push64_kernel(Push64Args A)
         }
         rhsT<double>(B0, g.a, eps, u[0], u[1], u[2], g.a * u[2], f0);
         double dt = A.dt;
-        double rt = fma(dt, f0.xr, r), tt = fma(dt, f0.xt, th), xpl = f0.xp;
-        double urt = fma(dt, f0.ur, u[0]), utt = fma(dt, f0.ut, u[1]);
         const double h = 0.5 * dt;
-        for (int it = 0; it < A.n_iter; ++it) {
+        double xpl = f0.xp;
+        double rt = fma(dt, f0.xr, r), tt = fma(dt, f0.xt, th);
+        double urt = fma(dt, f0.ur, u[0]), utt = fma(dt, f0.ut, u[1]);
+        int it = 0;
+        if constexpr (!TAPE) {
+            double dr, dth, dur, dut;
+            if (A.pairs && A.hf * float_of_pos(fabs(f0.xp)) < PAIR_MAX_ANGLE &&
+                correctors_df(A.a_df, A.a2_df, A.dt_df, A.n_iter - 1, (float)eps, r, s0, c0, u, f0, dr, dth, dur, dut)) {
+                rt = r + dr;
+                tt = th + dth;
+                urt = u[0] + dur;
+                utt = u[1] + dut;
+                it = A.n_iter - 1;
+            }
+        }
+        for (; it < A.n_iter; ++it) {
             // theta of the iterate within 0.05 of theta^n (the usual case: one
             // step moves a particle less than two cells): the series of
             // sincos_shift, truncated below 1e-17
@@ -469,6 +580,11 @@ static Push64Args push64_args(grpic_ctx *ctx, const grpic_particles *in, grpic_p
     A.idt = 1.0 / ctx->prm.dt;
     A.m_i2dt = -0.5 / ctx->prm.dt;
     A.n_iter = ctx->prm.n_push_iter;
+    A.pairs = A.n_iter >= 2 && A.dt <= PAIR_MAX_DT;
+    A.hf = (float)(0.5 * A.dt);
+    A.a_df = df_const(ctx->g.a);
+    A.a2_df = df_const(ctx->g.a * ctx->g.a);
+    A.dt_df = df_const(A.dt);
     for (int k = 0; k < 4; ++k) {
         A.qm[k] = ctx->prm.q_over_m[k];
         A.qw[k] = ctx->prm.q_weight[k];

@@ -85,3 +85,34 @@ def test_steps_keep_every_particle_and_its_order(nr, nth, r_in, r_out):
     assert np.array_equal(h["tag"], P.tag)
     assert np.median(np.abs(h["x1"] - P.r) / P.r) < 1e-13
     assert np.mean(np.abs(h["x2"] - P.th) < 1e-8) > 0.999
+
+
+@pytest.mark.parametrize("sigma", [0.05, 0.6])
+@pytest.mark.parametrize("n_iter", [1, 2, 3, 5])
+def test_correctors_in_pairs_keep_fp64(n_iter, sigma):
+    """The early correctors run in double-FP32 pairs where their error leaves the
+    last one under an eighth of a rounding (dt <= 0.02, off the axis).  Positions
+    then agree with the oracle's to a few roundings of FP64 (2^-53 = 1.1e-16; the
+    two push formulas round differently in about ten places of a step whose move
+    is at most 1e-2), near the axis, where FP64 takes over, included."""
+    from paper_2503_04558_gb300 import grpic as G
+    oc, gc = configs(128, 128, 0.9, 1.3, 50.0, n_push_iter=n_iter)
+    assert gc.dt <= 0.02
+    ctx = G.Context(gc)
+    F = G.Fields(gc)
+    ctx.init_fields(F, G.WALD, 1.0)
+    D, B = O.init_fields(oc, O.WALD, 1.0)
+    P = _particles(oc, 40000, 11)
+    f = sigma / 0.1
+    P.u1, P.u2, P.u3 = P.u1 * f, P.u2 * f, P.u3 * f
+    S = G.ParticleSet(gc, P.n)
+    S.load(P.r, P.th, P.u1, P.u2, P.u3, P.tag)
+    ctx.push(S, F)
+    st = ctx.sync()
+    so, J, _ = O.push_deposit(oc, P, D, B)
+    assert st == so
+    mid = np.abs(P.th - np.pi / 2) < 1.2
+    for k, ref, tol in (("x1", P.r, 2e-15), ("x2", P.th, 2e-15), ("u1", P.u1, 1e-13), ("u2", P.u2, 1e-13)):
+        got = getattr(S.a, k).cpu().numpy()
+        assert relerr(got[mid], ref[mid]) < tol, k
+        assert relerr(got, ref) < 1e-12, k
