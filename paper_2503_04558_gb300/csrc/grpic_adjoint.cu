@@ -163,236 +163,185 @@ __device__ void rhs_jac(double a, double eps, const double y[5], double F[5], do
     for (int k = 0; k < 5; ++k) dFp[k] = f[2].d[k];
 }
 
-// w^T dF/dy + wp dX^ph/dy at y = (r, th, u_r, u_th, u_ph) for F = (X^r, X^th,
-// U_r, U_th, 0), the right-hand side of Eq. particle-eom written as the push
-// evaluates it: with P = (a^2 + r^2) u_r^2 + 2 a u_r u_ph + u_th^2 +
-// u_ph^2 / sin^2,  u.u = P / rho^2 - beta u_r^2,  X^r = (g^rr u_r + g^rph u_ph)
-// / u^0 - beta,  Q_r = u_r^2 (z - d_r beta) - 2 r P / rho^4,  Q_th = -d_th rho^2
-// P / rho^4 - d_th beta u_r^2 - 2 sin cos u_ph^2 / (rho^2 sin^4),  U_i =
-// -alpha u^0 d_i alpha + u_r d_i beta - Q_i / (2 u^0).  The reverse pass runs
-// through those formulas; the r, theta (and a) derivatives of the thirteen
-// metric quantities they use come from dual numbers.  sv, cv = sin, cos y[1].
-template <int ND>
-__device__ void rhs_vjp_p(double a, double eps, const double y[5], double sv, double cv, const double w[5], double wp,
-                          double out[5], double *out_a = nullptr)
+// Adjoints of the point quantities of pointT (rho^2's inverse, z, 1 + z, its
+// inverse, beta, 1 / sin^2, a^2 + r^2, sin cos, E), collected by the reverse
+// passes below, and their transpose into r, theta (and a through a^2).
+struct PtAdj {
+    double ir, z, o, io, be, is2, A, cs, E;
+};
+__device__ __forceinline__ void point_vjp(const PtT<double> &m, double a2, double m2a2, double r, double c2, PtAdj L,
+                                          double Lrho2, double &Lr, double &Lth, double &La2)
 {
-    typedef DN<ND> D;
-    D r(y[0]), aD(a), s(sv), c(cv);
-    r.d[0] = 1.0;
-    s.d[1] = cv;
-    c.d[1] = -sv;
-    if constexpr (ND > 2) aD.d[2] = 1.0;
-    // metric quantities (dual)
-    const D a2 = aD * aD, r2 = r * r;
-    const D A2 = a2 + r2;
-    const D ir = rcp_t(r2 + a2 * c * c);
-    const D ir2 = ir * ir;
-    const D z = D(2.0) * r * ir;
-    const D iopz = rcp_t(D(1.0) + z);
-    const D alphaD = sqrt_t(iopz);
-    const D betaD = z * iopz;
-    const D is2 = rcp_t(s * s);
-    const D drho_t = D(-2.0) * a2 * c * s;
-    const D dz_r = D(2.0) * ir * (D(1.0) - D(2.0) * r2 * ir);
-    const D dz_t = D(-2.0) * r * drho_t * ir2;
-    const D ka = D(-0.5) * alphaD * iopz, kb = iopz * iopz;
-    const D da_r = ka * dz_r, da_t = ka * dz_t, db_r = kb * dz_r, db_t = kb * dz_t;
-    const D M2 = D(2.0) * r * ir2, M3 = drho_t * ir2, M4 = D(2.0) * s * c * ir * is2 * is2;
-    // forward values
-    const double ur = y[2], ut = y[3], up = y[4];
-    const double vA2 = A2.v, vir = ir.v, vbe = betaD.v, val = alphaD.v, vis2 = is2.v, vz = z.v;
-    const double ur2 = ur * ur, up2 = up * up;
-    const double P = vA2 * ur2 + 2.0 * a * ur * up + ut * ut + vis2 * up2;
-    const double uu = vir * P - vbe * ur2;
-    const double au0 = sqrt_t(eps + uu);
-    const double iau = rcp_t(au0);
-    const double iu0 = val * iau, h = 0.5 * iu0;
-    const double G1 = vA2 * vir - vbe, G2 = a * vir;
-    const double Qr = ur2 * (vz - db_r.v) - M2.v * P;
-    const double Qt = -M3.v * P - db_t.v * ur2 - M4.v * up2;
-    // reverse; adjoints of the outputs X^r, X^th, U_r, U_th, X^ph
-    const double Lxr = w[0], Lxt = w[1], Lur = w[2], Lut = w[3], Lxp = wp;
-    double L_ur = 0.0, L_ut = 0.0, L_up = 0.0, L_a = 0.0;
-    double L_A2 = 0.0, L_ir = 0.0, L_be = 0.0, L_al = 0.0, L_is2 = 0.0, L_z = 0.0;
-    double L_dar = 0.0, L_dat = 0.0, L_dbr = 0.0, L_dbt = 0.0, L_M2 = 0.0, L_M3 = 0.0, L_M4 = 0.0;
-    double L_au0 = 0.0, L_iu0 = 0.0, L_P = 0.0;
-    // U_r = -au0 da_r + ur db_r - h Qr,  U_th likewise
-    L_au0 -= Lur * da_r.v + Lut * da_t.v;
-    L_dar -= Lur * au0;
-    L_dat -= Lut * au0;
-    L_dbr += Lur * ur;
-    L_dbt += Lut * ur;
-    L_ur += Lur * db_r.v + Lut * db_t.v;
-    const double L_h = -Lur * Qr - Lut * Qt;
-    const double L_Qr = -Lur * h, L_Qt = -Lut * h;
-    // Qr = ur^2 (z - db_r) - M2 P
-    L_ur += L_Qr * 2.0 * ur * (vz - db_r.v);
-    L_z += L_Qr * ur2;
-    L_dbr -= L_Qr * ur2;
-    L_M2 -= L_Qr * P;
-    L_P -= L_Qr * M2.v;
-    // Qt = -M3 P - db_t ur^2 - M4 up^2
-    L_M3 -= L_Qt * P;
-    L_P -= L_Qt * M3.v;
-    L_dbt -= L_Qt * ur2;
-    L_ur -= L_Qt * 2.0 * db_t.v * ur;
-    L_M4 -= L_Qt * up2;
-    L_up -= L_Qt * 2.0 * M4.v * up;
-    // h = iu0 / 2
-    L_iu0 += 0.5 * L_h;
-    // X^r = (G1 ur + G2 up) iu0 - beta, G1 = A2 ir - beta, G2 = a ir
-    L_iu0 += Lxr * (G1 * ur + G2 * up);
-    L_ur += Lxr * G1 * iu0;
-    L_up += Lxr * G2 * iu0;
-    L_A2 += Lxr * ur * iu0 * vir;
-    L_ir += Lxr * iu0 * (ur * vA2 + a * up);
-    L_be -= Lxr * (ur * iu0 + 1.0);
-    L_a += Lxr * vir * up * iu0;
-    // X^th = ir ut iu0
-    L_iu0 += Lxt * vir * ut;
-    L_ut += Lxt * vir * iu0;
-    L_ir += Lxt * ut * iu0;
-    // X^ph = (a ir ur + ir is2 up) iu0
-    L_iu0 += Lxp * (a * vir * ur + vir * vis2 * up);
-    L_ur += Lxp * a * vir * iu0;
-    L_up += Lxp * vir * vis2 * iu0;
-    L_ir += Lxp * (a * ur + vis2 * up) * iu0;
-    L_is2 += Lxp * vir * up * iu0;
-    L_a += Lxp * vir * ur * iu0;
-    // iu0 = alpha / au0, au0 = sqrt(eps + uu)
-    L_al += L_iu0 * iau;
-    L_au0 -= L_iu0 * val * iau * iau;
-    const double L_uu = 0.5 * L_au0 * iau;
-    // uu = ir P - beta ur^2
-    L_ir += L_uu * P;
-    L_P += L_uu * vir;
-    L_be -= L_uu * ur2;
-    L_ur -= L_uu * 2.0 * vbe * ur;
-    // P = A2 ur^2 + 2 a ur up + ut^2 + is2 up^2
-    L_A2 += L_P * ur2;
-    L_ur += L_P * (2.0 * vA2 * ur + 2.0 * a * up);
-    L_up += L_P * (2.0 * a * ur + 2.0 * vis2 * up);
-    L_ut += L_P * 2.0 * ut;
-    L_is2 += L_P * up2;
-    L_a += L_P * 2.0 * ur * up;
-    // metric quantities -> r, theta (and a)
-    const D *q[13] = {&A2, &ir, &betaD, &alphaD, &is2, &z, &da_r, &da_t, &db_r, &db_t, &M2, &M3, &M4};
-    const double Lq[13] = {L_A2, L_ir, L_be, L_al, L_is2, L_z, L_dar, L_dat, L_dbr, L_dbt, L_M2, L_M3, L_M4};
-    double Lr = 0.0, Lth = 0.0;
-#pragma unroll
-    for (int k = 0; k < 13; ++k) {
-        Lr += Lq[k] * q[k]->d[0];
-        Lth += Lq[k] * q[k]->d[1];
-    }
-    if constexpr (ND > 2) {
-        double La = L_a;
-#pragma unroll
-        for (int k = 0; k < 13; ++k) La += Lq[k] * q[k]->d[2];
-        *out_a += La;
-    }
-    out[0] = Lr;
-    out[1] = Lth;
-    out[2] = L_ur;
-    out[3] = L_ut;
-    out[4] = L_up;
+    // E = -2 a^2 sin cos / rho^2
+    const double e = m2a2 * L.E;
+    L.cs = fma(e, m.ir, L.cs);
+    L.ir = fma(e, m.cs, L.ir);
+    // beta = z / (1 + z), 1 / (1 + z), z = 2 r / rho^2
+    L.z = fma(L.be, m.iopz, L.z);
+    L.io = fma(L.be, m.z, L.io);
+    L.z += fma(-L.io, m.iopz * m.iopz, L.o);
+    L.ir = fma(L.z, r + r, L.ir);
+    // 1 / rho^2, rho^2 = r^2 + a^2 cos^2, a^2 + r^2
+    const double R = fma(-L.ir, m.ir * m.ir, Lrho2);
+    Lr = fma(r + r, R + L.A, (L.z + L.z) * m.ir);
+    // d cos^2 = -2 sin cos, d (sin cos) = cos^2 - sin^2, d sin^-2 = -2 sin cos / sin^4
+    const double k = m.cs * m.is2;
+    Lth = fma(L.cs, c2 - m.s2, fma(m2a2 * m.cs, R, -(L.is2 + L.is2) * (k * m.is2)));
+    La2 = fma(R, c2, fma(-2.0 * m.cs * m.ir, L.E, L.A));
+}
+
+// w^T dF/dy + wp dX^ph/dy at y = (r, th, u_r, u_th, u_ph) for F = (X^r, X^th,
+// U_r, U_th, 0): the reverse pass through the right-hand side exactly as the push
+// evaluates it (pointT and rhsT), about 165 FP64 operations.  (Through dual
+// numbers in r and theta for thirteen metric quantities: about 350.)  out_a
+// (ND = 3) receives the part through the spin.  sv, cv = sin, cos y[1].
+template <int ND>
+__device__ __forceinline__ void rhs_vjp_p(double a, double eps, const double y[5], double sv, double cv,
+                                          const double w[5], double wp, double out[5], double *out_a = nullptr)
+{
+    double a2 = a * a, m2a2 = -2.0 * a2, r = y[0], ur = y[2], ut = y[3], up = y[4], aup = a * up;
+    const PtT<double> m = pointT<double>(a2, m2a2, r, sv, cv);
+    // forward (rhsT)
+    double ur2 = ur * ur, p = m.is2 * up, p2 = p * up;
+    double W = fma(m.ar2, ur, aup), P = fma(ur, W + aup, fma(ut, ut, p2));
+    double I = m.ir * P, Q = fma(-m.beta, ur2, I + eps);
+    double iu = rsqrt_fast(m.opz * Q), h = 0.5 * iu, ii = m.ir * iu;
+    double T1 = m.iopz * ur, T2 = fma(h, ur, 1.0), T = fma(T1, T2, h * Q), K = m.iopz * T;
+    double B2 = I - ur2, B4 = m.cs * m.is2;
+    // reverse: U_r = K (2 / rho^2 - z^2) + h z B2, U_th = E (h I - K z) + ii B4 p2,
+    // X^r = iu (ir W - beta u_r) - beta, X^th = ii u_th, X^ph = ii (a u_r + p)
+    double Lr = w[2], Lt = w[3];
+    double rK = Lr * K, tE = Lt * m.E, rh = Lr * h;
+    PtAdj L;
+    double LK = fma(Lr, fma(-m.z, m.z, m.ir + m.ir), -tE * m.z);
+    L.z = fma(rh, B2, fma(-(m.z + m.z), rK, -tE * K));
+    double Lh = fma(Lr * m.z, B2, tE * I);
+    double rhz = rh * m.z;
+    double LI = fma(tE, h, rhz);
+    L.E = Lt * fma(h, I, -K * m.z);
+    double tp2 = Lt * p2;
+    double Lii = fma(tp2, B4, fma(w[1], ut, wp * fma(a, ur, p)));
+    double b4 = tp2 * ii;
+    L.cs = b4 * m.is2;
+    L.is2 = b4 * m.cs;
+    double Lp2 = Lt * ii * B4;
+    double Lut = w[1] * ii;
+    double pii = wp * ii;
+    double V = w[0] * iu;
+    double Liu = w[0] * fma(m.ir, W, -m.beta * ur);
+    double Lw = V * m.ir;
+    L.be = -fma(V, ur, w[0]);
+    double Lur = fma(pii, a, fma(-V, m.beta, -2.0 * rhz * ur));
+    // K = T / (1 + z), T = T1 T2 + h Q
+    double LT = LK * m.iopz;
+    L.io = fma(LK, T, LT * ur * T2);
+    Lur = fma(LT, fma(T1, h, m.iopz * T2), Lur);
+    Lh = fma(LT, fma(T1, ur, Q), Lh);
+    double LQ = LT * h;
+    // ii = ir iu, h = iu / 2, iu = ((1 + z) Q)^-1/2
+    L.ir = fma(Lii, iu, fma(V, W, rK + rK));
+    Liu = fma(Lii, m.ir, fma(0.5, Lh, Liu));
+    double G = -h * iu * iu * Liu;
+    L.o = G * Q;
+    LQ = fma(G, m.opz, LQ);
+    // Q = I - beta u_r^2 + eps, I = P / rho^2, P = u_r (W + a u_ph) + u_th^2 + p2
+    LI += LQ;
+    L.be = fma(-LQ, ur2, L.be);
+    L.ir = fma(LI, P, L.ir);
+    double LP = LI * m.ir;
+    Lw = fma(LP, ur, Lw);
+    Lur = fma(-2.0 * LQ * m.beta, ur, fma(LP, W + aup, Lur));
+    Lur = fma(Lw, m.ar2, Lur);
+    Lut = fma(LP + LP, ut, Lut);
+    Lp2 += LP;
+    L.A = Lw * ur;
+    // p2 = p u_ph, p = u_ph / sin^2
+    double Lp = fma(Lp2, up, pii);
+    L.is2 = fma(Lp, up, L.is2);
+    out[2] = Lur;
+    out[3] = Lut;
+    out[4] = fma(Lp2, p, fma(Lp, m.is2, a * fma(LP, ur, Lw)));
+    double La2;
+    point_vjp(m, a2, m2a2, r, cv * cv, L, 0.0, out[0], out[1], La2);
+    if constexpr (ND > 2) *out_a += fma(2.0 * a, La2, fma(pii, ur, up * fma(LP, ur, Lw)));
 }
 
 // lo^T d(u')/dz for the generalized Boris step (Eqs. boris-plus-minus, u0bar,
 // boris-scheme) u' = u'(z), z = (r, th, u_r, u_th, u_ph, D^r, D^th, D^ph, B^r,
-// B^th, B^ph): its reverse pass written out by hand, the metric's r and theta
-// derivatives from two-slot dual numbers; sn, cs = sin, cos of theta
+// B^th, B^ph): its reverse pass written out by hand, the metric's through the
+// point quantities; sn, cs = sin, cos of theta
 template <int ND>
-__device__ void boris_vjp(double a, double qm, double dt, const double z[11], double sn, double cs, const double lo[3],
-                          double out[11], double *out_a = nullptr)
+__device__ __forceinline__ void boris_vjp(double a, double qm, double dt, const double z[11], double sn, double cs,
+                                          const double lo[3], double out[11], double *out_a = nullptr)
 {
-    // slots: d/dr, d/dtheta (and d/da when ND = 3)
-    DN<ND> r(z[0]), aD(a), s(sn), c(cs);
-    r.d[0] = 1.0;
-    s.d[1] = cs;
-    c.d[1] = -sn;
-    if constexpr (ND > 2) aD.d[2] = 1.0;
-    const DN<ND> a2 = aD * aD, s2 = s * s;
-    const DN<ND> rho2 = r * r + a2 * c * c;
-    const DN<ND> ir = rcp_t(rho2);
-    const DN<ND> zz = DN<ND>(2.0) * r * ir;
-    const DN<ND> opz = DN<ND>(1.0) + zz;
-    const DN<ND> alphaD = sqrt_t(rcp_t(opz));
-    const DN<ND> Dl_ = r * r + a2 - DN<ND>(2.0) * r;
-    const DN<ND> Sg = (r * r + a2) * (r * r + a2) - a2 * Dl_ * s2;
-    // metric quantities q[] = g_rr, g_rp, g_tt, g_pp, i_rr, i_rp, i_tt, i_pp, sqrt(gamma), alpha
-    DN<ND> q[10];
-    q[0] = opz;
-    q[1] = -aD * s2 * opz;
-    q[2] = rho2;
-    q[3] = Sg * s2 * ir;
-    q[4] = (a2 + r * r) * ir - zz * rcp_t(opz);
-    q[5] = aD * ir;
-    q[6] = ir;
-    q[7] = ir * rcp_t(s2);
-    q[8] = rho2 * s * sqrt_t(opz);
-    q[9] = alphaD;
-    const double grr = q[0].v, grp = q[1].v, gtt = q[2].v, gpp = q[3].v;
-    const double irr = q[4].v, irp = q[5].v, itt = q[6].v, ipp = q[7].v, sg = q[8].v, alpha = q[9].v;
-    const double u[3] = {z[2], z[3], z[4]}, D[3] = {z[5], z[6], z[7]}, B[3] = {z[8], z[9], z[10]};
-    const double c1 = 0.5 * qm * dt;
+    // (not const: the host compiler front end folds chains of const doubles in
+    // time exponential in their length)
+    double a2 = a * a, m2a2 = -2.0 * a2, r = z[0];
+    const PtT<double> m = pointT<double>(a2, m2a2, r, sn, cs);
+    double alpha = lapse(m);
+    double gz = fma(m.z * a2, m.s2, m.ar2);  // g_pp = sin^2 (a^2 + r^2 + z a^2 sin^2)
+    double as2 = a * m.s2, sgo = m.rho2 * sn;
+    double grr = m.opz, grp = -as2 * m.opz, gtt = m.rho2, gpp = m.s2 * gz;
+    double irr = fma(m.ar2, m.ir, -m.beta), irp = a * m.ir, itt = m.ir, ipp = m.ir * m.is2;
+    double oa = m.opz * alpha;               // sqrt(1 + z)
+    double sg = sgo * oa;
+    double u[3] = {z[2], z[3], z[4]}, D[3] = {z[5], z[6], z[7]}, B[3] = {z[8], z[9], z[10]};
+    double c1 = 0.5 * qm * dt;
     // forward values
-    const double Dl[3] = {grr * D[0] + grp * D[2], gtt * D[1], grp * D[0] + gpp * D[2]};
-    const double h = c1 * alpha;
-    const double um[3] = {u[0] + h * Dl[0], u[1] + h * Dl[1], u[2] + h * Dl[2]};
-    const double v[3] = {irr * um[0] + irp * um[2], itt * um[1], irp * um[0] + ipp * um[2]};
-    const double S = 1.0 + um[0] * v[0] + um[1] * v[1] + um[2] * v[2];
-    const double rS = sqrt_t(S);
-    const double ialpha = rcp_t(alpha), irS = rcp_t(rS);
-    const double u0b = rS * ialpha;
-    const double iu0b = alpha * irS;
-    const double kt = c1 * iu0b;
-    const double t[3] = {kt * B[0], kt * B[1], kt * B[2]};
-    const double Gt[3] = {grr * t[0] + grp * t[2], gtt * t[1], grp * t[0] + gpp * t[2]};
-    const double tt = t[0] * Gt[0] + t[1] * Gt[1] + t[2] * Gt[2];
-    const double i1tt = rcp_t(1.0 + tt);
-    const double ks = 2.0 * i1tt;
-    const double sv[3] = {ks * t[0], ks * t[1], ks * t[2]};
-    const double vt[3] = {v[1] * t[2] - v[2] * t[1], v[2] * t[0] - v[0] * t[2], v[0] * t[1] - v[1] * t[0]};
-    const double w[3] = {um[0] + sg * vt[0], um[1] + sg * vt[1], um[2] + sg * vt[2]};
-    const double x[3] = {irr * w[0] + irp * w[2], itt * w[1], irp * w[0] + ipp * w[2]};
-    const double C[3] = {x[1] * sv[2] - x[2] * sv[1], x[2] * sv[0] - x[0] * sv[2], x[0] * sv[1] - x[1] * sv[0]};
-    // reverse: out_i = um_i + sg C_i + h Dl_i
+    double Dl[3] = {grr * D[0] + grp * D[2], gtt * D[1], grp * D[0] + gpp * D[2]};
+    double h = c1 * alpha;
+    double um[3] = {u[0] + h * Dl[0], u[1] + h * Dl[1], u[2] + h * Dl[2]};
+    double v[3] = {irr * um[0] + irp * um[2], itt * um[1], irp * um[0] + ipp * um[2]};
+    double S = 1.0 + um[0] * v[0] + um[1] * v[1] + um[2] * v[2];
+    double irS = rsqrt_fast(S);
+    double iu0b = alpha * irS;               // 1 / u0bar
+    double kt = c1 * iu0b;
+    double t[3] = {kt * B[0], kt * B[1], kt * B[2]};
+    double Gt[3] = {grr * t[0] + grp * t[2], gtt * t[1], grp * t[0] + gpp * t[2]};
+    double tt = t[0] * Gt[0] + t[1] * Gt[1] + t[2] * Gt[2];
+    double i1tt = rcp_t(1.0 + tt);
+    double ks = 2.0 * i1tt;
+    double sv[3] = {ks * t[0], ks * t[1], ks * t[2]};
+    double vt[3] = {v[1] * t[2] - v[2] * t[1], v[2] * t[0] - v[0] * t[2], v[0] * t[1] - v[1] * t[0]};
+    double w[3] = {um[0] + sg * vt[0], um[1] + sg * vt[1], um[2] + sg * vt[2]};
+    double x[3] = {irr * w[0] + irp * w[2], itt * w[1], irp * w[0] + ipp * w[2]};
+    double C[3] = {x[1] * sv[2] - x[2] * sv[1], x[2] * sv[0] - x[0] * sv[2], x[0] * sv[1] - x[1] * sv[0]};
+    // reverse: out_i = um_i + sg C_i + h Dl_i; the metric's adjoints
+    double Lgrr, Lgrp, Lgtt, Lgpp, Lirr, Lirp, Litt, Lipp, Lsg, Lal;
     double Lum[3] = {lo[0], lo[1], lo[2]};
     double Lh = lo[0] * Dl[0] + lo[1] * Dl[1] + lo[2] * Dl[2];
     double LDl[3] = {lo[0] * h, lo[1] * h, lo[2] * h};
-    double Lq[10] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
-    Lq[8] += lo[0] * C[0] + lo[1] * C[1] + lo[2] * C[2];
-    const double LC[3] = {lo[0] * sg, lo[1] * sg, lo[2] * sg};
+    Lsg = lo[0] * C[0] + lo[1] * C[1] + lo[2] * C[2];
+    double LC[3] = {lo[0] * sg, lo[1] * sg, lo[2] * sg};
     // C = x cross s
     double Lx[3] = {sv[1] * LC[2] - sv[2] * LC[1], sv[2] * LC[0] - sv[0] * LC[2], sv[0] * LC[1] - sv[1] * LC[0]};
     double Ls[3] = {LC[1] * x[2] - LC[2] * x[1], LC[2] * x[0] - LC[0] * x[2], LC[0] * x[1] - LC[1] * x[0]};
     // x = Ginv w
     double Lw[3] = {irr * Lx[0] + irp * Lx[2], itt * Lx[1], irp * Lx[0] + ipp * Lx[2]};
-    Lq[4] += Lx[0] * w[0];
-    Lq[5] += Lx[0] * w[2] + Lx[2] * w[0];
-    Lq[6] += Lx[1] * w[1];
-    Lq[7] += Lx[2] * w[2];
+    Lirr = Lx[0] * w[0];
+    Lirp = Lx[0] * w[2] + Lx[2] * w[0];
+    Litt = Lx[1] * w[1];
+    Lipp = Lx[2] * w[2];
     // w = um + sg (v cross t)
     for (int i = 0; i < 3; ++i) Lum[i] += Lw[i];
-    Lq[8] += Lw[0] * vt[0] + Lw[1] * vt[1] + Lw[2] * vt[2];
-    const double LD_[3] = {Lw[0] * sg, Lw[1] * sg, Lw[2] * sg};
+    Lsg += Lw[0] * vt[0] + Lw[1] * vt[1] + Lw[2] * vt[2];
+    double LD_[3] = {Lw[0] * sg, Lw[1] * sg, Lw[2] * sg};
     double Lv[3] = {t[1] * LD_[2] - t[2] * LD_[1], t[2] * LD_[0] - t[0] * LD_[2], t[0] * LD_[1] - t[1] * LD_[0]};
     double Lt[3] = {LD_[1] * v[2] - LD_[2] * v[1], LD_[2] * v[0] - LD_[0] * v[2], LD_[0] * v[1] - LD_[1] * v[0]};
     // s = ks t, ks = 2 / (1 + tt), tt = t^T G t
-    const double Lks = Ls[0] * t[0] + Ls[1] * t[1] + Ls[2] * t[2];
+    double Lks = Ls[0] * t[0] + Ls[1] * t[1] + Ls[2] * t[2];
     for (int i = 0; i < 3; ++i) Lt[i] += ks * Ls[i];
-    const double Ltt = -Lks * 2.0 * i1tt * i1tt;
+    double Ltt = -Lks * 2.0 * i1tt * i1tt;
     for (int i = 0; i < 3; ++i) Lt[i] += 2.0 * Ltt * Gt[i];
-    Lq[0] += Ltt * t[0] * t[0];
-    Lq[1] += Ltt * 2.0 * t[0] * t[2];
-    Lq[2] += Ltt * t[1] * t[1];
-    Lq[3] += Ltt * t[2] * t[2];
-    // t = kt B, kt = c1 / u0b, u0b = sqrt(S) / alpha
-    const double Lkt = Lt[0] * B[0] + Lt[1] * B[1] + Lt[2] * B[2];
-    const double LB[3] = {kt * Lt[0], kt * Lt[1], kt * Lt[2]};
-    const double Lu0b = -Lkt * c1 * iu0b * iu0b;
-    const double LS = 0.5 * Lu0b * irS * ialpha;
-    Lq[9] -= Lu0b * rS * ialpha * ialpha;
+    Lgrr = Ltt * t[0] * t[0];
+    Lgrp = Ltt * 2.0 * t[0] * t[2];
+    Lgtt = Ltt * t[1] * t[1];
+    Lgpp = Ltt * t[2] * t[2];
+    // t = kt B, kt = c1 alpha / sqrt(S)
+    double Lkt = Lt[0] * B[0] + Lt[1] * B[1] + Lt[2] * B[2];
+    double LB[3] = {kt * Lt[0], kt * Lt[1], kt * Lt[2]};
+    Lal = Lkt * c1 * irS;
+    double LS = -0.5 * Lkt * kt * irS * irS;
     // S = 1 + um . v, v = Ginv um
     for (int i = 0; i < 3; ++i) {
         Lum[i] += LS * v[i];
@@ -401,35 +350,38 @@ __device__ void boris_vjp(double a, double qm, double dt, const double z[11], do
     Lum[0] += irr * Lv[0] + irp * Lv[2];
     Lum[1] += itt * Lv[1];
     Lum[2] += irp * Lv[0] + ipp * Lv[2];
-    Lq[4] += Lv[0] * um[0];
-    Lq[5] += Lv[0] * um[2] + Lv[2] * um[0];
-    Lq[6] += Lv[1] * um[1];
-    Lq[7] += Lv[2] * um[2];
+    Lirr += Lv[0] * um[0];
+    Lirp += Lv[0] * um[2] + Lv[2] * um[0];
+    Litt += Lv[1] * um[1];
+    Lipp += Lv[2] * um[2];
     // um = u + h Dl, h = c1 alpha, Dl = G D
     for (int i = 0; i < 3; ++i) {
         Lh += Lum[i] * Dl[i];
         LDl[i] += h * Lum[i];
     }
-    Lq[9] += c1 * Lh;
-    const double LDv[3] = {grr * LDl[0] + grp * LDl[2], gtt * LDl[1], grp * LDl[0] + gpp * LDl[2]};
-    Lq[0] += LDl[0] * D[0];
-    Lq[1] += LDl[0] * D[2] + LDl[2] * D[0];
-    Lq[2] += LDl[1] * D[1];
-    Lq[3] += LDl[2] * D[2];
-    double Lr = 0.0, Lth = 0.0;
-#pragma unroll
-    for (int k = 0; k < 10; ++k) {
-        Lr += Lq[k] * q[k].d[0];
-        Lth += Lq[k] * q[k].d[1];
-    }
-    if constexpr (ND > 2) {
-        double La = 0.0;
-#pragma unroll
-        for (int k = 0; k < 10; ++k) La += Lq[k] * q[k].d[2];
-        *out_a += La;
-    }
-    out[0] = Lr;
-    out[1] = Lth;
+    Lal += c1 * Lh;
+    double LDv[3] = {grr * LDl[0] + grp * LDl[2], gtt * LDl[1], grp * LDl[0] + gpp * LDl[2]};
+    Lgrr += LDl[0] * D[0];
+    Lgrp += LDl[0] * D[2] + LDl[2] * D[0];
+    Lgtt += LDl[1] * D[1];
+    Lgpp += LDl[2] * D[2];
+    // the metric from the point quantities: sqrt(gamma) = rho^2 sin sqrt(1 + z), alpha =
+    // (1 + z)^-1/2, gamma_rph = -a sin^2 (1 + z), gamma_phph = sin^2 gz and the upper one
+    PtAdj L;
+    L.o = Lgrr - as2 * Lgrp + 0.5 * (Lsg * sgo * alpha - Lal * alpha * m.iopz);
+    double Lgz = Lgpp * m.s2;
+    L.A = Lgz + Lirr * m.ir;
+    L.z = Lgz * a2 * m.s2;
+    L.be = -Lirr;
+    L.ir = Lirr * m.ar2 + Lirp * a + Litt + Lipp * m.is2;
+    L.is2 = Lipp * m.ir;
+    L.io = L.cs = L.E = 0.0;
+    double Lrho2 = Lgtt + Lsg * sn * oa;
+    double Ls2 = Lgpp * gz + Lgz * m.z * a2 - Lgrp * a * m.opz;  // through sin^2
+    double La2;
+    point_vjp(m, a2, m2a2, r, cs * cs, L, Lrho2, out[0], out[1], La2);
+    out[1] += 2.0 * m.cs * Ls2 + Lsg * m.rho2 * oa * cs;
+    if constexpr (ND > 2) *out_a += 2.0 * a * (La2 + Lgz * m.z * m.s2) + Lirp * m.ir - Lgrp * m.s2 * m.opz;
     for (int i = 0; i < 3; ++i) {
         out[2 + i] = Lum[i];
         out[5 + i] = LDv[i];
