@@ -420,60 +420,39 @@ __device__ void solve5(double M[5][5], double b[5])
     }
 }
 
-__device__ __forceinline__ double W1(double d)
-{
-    d = fabs(d);
-    return d < 1.0 ? 1.0 - d : 0.0;
-}
-__device__ __forceinline__ double dW1(double d) { return fabs(d) < 1.0 ? (d > 0.0 ? -1.0 : (d < 0.0 ? 1.0 : 0.0)) : 0.0; }
-
-// staggered bilinear stencil with axis mirroring (as in the push)
+// a component's bilinear stencil (as the push's gather): column and rows of the
+// corners, offsets, mirror rows of an odd component
 struct St {
     int c0, r0, r1;
-    double f, gg, p0, p1;
+    double f, gg;
+    bool flip0, flip1;
 };
-__device__ __forceinline__ void stencil(const GridDev &g, double x1, double x2, bool half_r, bool half_t, double par,
-                                        St &S)
-{
-    double xi = half_r ? x1 - 0.5 : x1;
-    double fi = floor(xi);
-    S.f = xi - fi;
-    S.c0 = (int)fi + NG;
-    S.p0 = S.p1 = 1.0;
-    if (half_t) {
-        double eta = x2 - 0.5, fj = floor(eta);
-        int j = (int)fj;
-        S.gg = eta - fj;
-        S.r0 = j;
-        S.r1 = j + 1;
-        if (S.r0 < 0) { S.r0 = -1 - S.r0; S.p0 = par; }
-        if (S.r1 > g.nth - 1) { S.r1 = 2 * g.nth - 1 - S.r1; S.p1 = par; }
-    } else {
-        int j = (int)floor(x2);
-        if (j > g.nth - 1) j = g.nth - 1;
-        S.gg = x2 - j;
-        S.r0 = j;
-        S.r1 = j + 1;
-    }
-}
 // value and d/dx1, d/dx2 (logical) of the interpolant
 __device__ __forceinline__ void gather_d(const double *F, int64_t ld, const St &S, double &v, double &d1, double &d2)
 {
-    double a00 = S.p0 * F[(size_t)S.r0 * ld + S.c0], a10 = S.p0 * F[(size_t)S.r0 * ld + S.c0 + 1];
-    double a01 = S.p1 * F[(size_t)S.r1 * ld + S.c0], a11 = S.p1 * F[(size_t)S.r1 * ld + S.c0 + 1];
-    double f = S.f, g = S.gg;
-    v = (1 - f) * (1 - g) * a00 + f * (1 - g) * a10 + (1 - f) * g * a01 + f * g * a11;
-    d1 = (1 - g) * (a10 - a00) + g * (a11 - a01);
-    d2 = (1 - f) * (a01 - a00) + f * (a11 - a10);
+    const double *a = F + (size_t)S.r0 * ld + S.c0, *b = F + (size_t)S.r1 * ld + S.c0;
+    double a0 = flip_sign(__ldg(a), S.flip0), b0 = flip_sign(__ldg(b), S.flip1);
+    double da = flip_sign(__ldg(a + 1), S.flip0) - a0, db = flip_sign(__ldg(b + 1), S.flip1) - b0;
+    double x = fma(S.f, da, a0);
+    d2 = fma(S.f, db, b0) - x;
+    v = fma(S.gg, d2, x);
+    d1 = fma(S.gg, db - da, da);
 }
 __device__ __forceinline__ void scatter_w(double *L, int64_t ld, const St &S, double lam)
 {
-    double f = S.f, g = S.gg;
-    atomicAdd(L + (size_t)S.r0 * ld + S.c0, S.p0 * (1 - f) * (1 - g) * lam);
-    atomicAdd(L + (size_t)S.r0 * ld + S.c0 + 1, S.p0 * f * (1 - g) * lam);
-    atomicAdd(L + (size_t)S.r1 * ld + S.c0, S.p1 * (1 - f) * g * lam);
-    atomicAdd(L + (size_t)S.r1 * ld + S.c0 + 1, S.p1 * f * g * lam);
+    double *a = L + (size_t)S.r0 * ld + S.c0, *b = L + (size_t)S.r1 * ld + S.c0;
+    double hi = S.gg * lam, lo = lam - hi, fl = S.f * lo, fh = S.f * hi;
+    atomicAdd(a, flip_sign(lo - fl, S.flip0));
+    atomicAdd(a + 1, flip_sign(fl, S.flip0));
+    atomicAdd(b, flip_sign(hi - fh, S.flip1));
+    atomicAdd(b + 1, flip_sign(fh, S.flip1));
 }
+
+// two neighbouring values along one dimension: their interpolant and difference
+struct Pair2 {
+    double v, d;
+};
+__device__ __forceinline__ Pair2 pair_at(double a, double b, double f) { return {fma(f, b - a, a), b - a}; }
 
 constexpr int MAX_ITER = 16;  // correctors the adjoint accepts
 
@@ -518,14 +497,14 @@ __global__ void __launch_bounds__(128) particle_adjoint(PAdjArgs A)
     double r = A.x[0][p], th = A.x[1][p];
     double u[3] = {A.x[2][p], A.x[3][p], A.x[4][p]};
     // a state the push refused (outside the domain, non-finite) moved nothing
-    bool inside = isfinite(r) && isfinite(th) && isfinite(u[0]) && isfinite(u[1]) && isfinite(u[2]) &&
-                  r >= g.r_in && r < g.r_out && th >= 0.0 && th <= M_PI;
+    bool inside = finite64(r) && finite64(th) && finite64(u[0]) && finite64(u[1]) && finite64(u[2]) && r >= g.r_in &&
+                  r < g.r_out && th >= 0.0 && th <= M_PI;
     if (!inside) {
         for (int k = 0; k < 5; ++k) A.lam0[k][p] = 0.0;
         return;
     }
     const ColPos ca = r_column_in(g, r);  // as in the push
-    const double x1a = ca.i + ca.f, x2a = theta_cells(g, th);
+    const double x2a = theta_cells(g, th);
     const double dt = A.dt, eps = massive ? 1.0 : 0.0;
     // the forward push's record: u' after the Boris step, the corrector
     // iterates, x^{n+1} before the reflection
@@ -541,12 +520,14 @@ __global__ void __launch_bounds__(128) particle_adjoint(PAdjArgs A)
     if (th1 < 0.0) { th1 = -th1; refl = -1.0; }
     else if (th1 > M_PI) { th1 = 2.0 * M_PI - th1; refl = -1.0; }
     const ColPos cb = r_column(g, y1[0]);
-    const double x1b = cb.i + cb.f, x2b = theta_cells(g, th1);
-    const int i0 = ca.i, j0 = row_of(g, x2a);
-    const int di = cb.i - i0, dj = row_of(g, x2b) - j0;
+    const double x2b = theta_cells(g, th1);
+    const int i0 = ca.i, j0 = row_of(g, x2a), j1 = row_of(g, x2b);
+    const int di = cb.i - i0, dj = j1 - j0;
+    // offsets of the start and end points in their cells
+    const double fa1 = ca.f, fa2 = x2a - j0, fb1 = cb.f, fb2 = x2b - j1;
     // the push's own checks: a finite end point, at most one cell away
-    bool moved_ok = di >= -1 && di <= 1 && dj >= -1 && dj <= 1 && y1[0] > 0.0 && isfinite(y1[0]) && isfinite(x2b) &&
-                    isfinite(y1[2]) && isfinite(y1[3]) && isfinite(dphi);
+    bool moved_ok = di >= -1 && di <= 1 && dj >= -1 && dj <= 1 && y1[0] > 0.0 && finite64(y1[0]) && finite64(x2b) &&
+                    finite64(y1[2]) && finite64(y1[3]) && finite64(dphi);
     if (!moved_ok) {
         for (int k = 0; k < 5; ++k) A.lam0[k][p] = 0.0;
         return;
@@ -559,88 +540,93 @@ __global__ void __launch_bounds__(128) particle_adjoint(PAdjArgs A)
     double ldphi = 0.0, lx1a = 0.0, lx2a = 0.0, lx1b = 0.0, lx2b = 0.0;
     double qw = A.qw[sp];
     if (qw != 0.0) {
-        // transpose of the Esirkepov window (same algebra as the push), each
-        // current's window contracted with its adjoint one row or column at a
-        // time: J^r A_r(k+1/2, l) = cr P_r(k) (S1_t + S0_t)(l), J^th A_th
-        // likewise, J^phi dV(k, l) = cq dphi (S1_r A_t + S0_r B_t)(k, l) with
-        // A_t = S1_t / 3 + S0_t / 6, B_t = S1_t / 6 + S0_t / 3
-        double S0r[4], S1r[4], S0t[4], S1t[4], dS0r[4], dS1r[4], dS0t[4], dS1t[4];
-        for (int k = 0; k < 4; ++k) {
-            double cr_ = i0 - 1 + k, ct = j0 - 1 + k;
-            S0r[k] = W1(x1a - cr_); dS0r[k] = dW1(x1a - cr_);
-            S1r[k] = W1(x1b - cr_); dS1r[k] = dW1(x1b - cr_);
-            S0t[k] = W1(x2a - ct); dS0t[k] = dW1(x2a - ct);
-            S1t[k] = W1(x2b - ct); dS1t[k] = dW1(x2b - ct);
-        }
-        const double cr = -qw / (2.0 * dt), cq = qw / dt, cp = cq * dphi;
-        const double c3 = 1.0 / 3.0, c6 = 1.0 / 6.0;
-        double Pr = 0.0, dPr1 = 0.0, dPr0 = 0.0;
-        for (int k = 0; k < 3; ++k) {
-            Pr += S1r[k] - S0r[k];
-            dPr1 += dS1r[k];
-            dPr0 += dS0r[k];
-            double U = 0.0, V = 0.0, W = 0.0;
-            for (int l = 0; l < 4; ++l) {
-                int row = j0 - 1 + l;
-                if (row < 0 || row > g.nth) continue;
-                double L = A.lamJ[0][(size_t)row * A.ld + (i0 - 1 + k + NG)];
-                U += L * (S1t[l] + S0t[l]);
-                V += L * dS1t[l];
-                W += L * dS0t[l];
+        // Transpose of the Esirkepov window.  The start's weights are (1 - f, f) at the
+        // nodes of its cell (columns / rows 1, 2 of the window), the end's at those of
+        // its own (di, dj cells on), so a current's window contracted with its adjoint L
+        // is interpolation of L:
+        //   J^r A_r at face k: cr P_r(k) (L interpolated in theta at the start + at the
+        //   end), P_r nonzero at face 1 and, for a move in r, at the extra face, and
+        //   P_r's derivatives -1 at the start's and the end's own face;
+        //   J^theta A_theta likewise; J^phi dV: cp (I_11 / 3 + (I_10 + I_01) / 6 + I_00 / 3),
+        //   I_pq bilinear with the end's (1) or start's (0) weights in r (p) and theta (q).
+        // At a node itself (offset 0) the weights' derivative is taken as 0.
+        double cr = -0.5 * qw / dt, cq = qw / dt, cp = cq * dphi;
+        const size_t w0 = (size_t)j0 * A.ld + (i0 + NG);  // the start cell's node
+        const size_t w1 = (size_t)j1 * A.ld + (i0 + di + NG);
+        const int64_t ld = A.ld;
+        {   // J^r: rows j0, j0 + 1 (start) and j1, j1 + 1 (end) at a face's column
+            const double *L = A.lamJ[0];
+            auto face = [&](int c, Pair2 &a, Pair2 &b) {
+                const double *s0 = L + (w0 + c), *s1 = L + (w0 + (int64_t)dj * ld + c);
+                a = pair_at(__ldg(s0), __ldg(s0 + ld), fa2);
+                b = pair_at(__ldg(s1), __ldg(s1 + ld), fb2);
+            };
+            Pair2 a, b;
+            face(0, a, b);
+            double P = cr * (fa1 - (di == 0 ? fb1 : (di > 0 ? 1.0 : 0.0))), U = cr * (a.v + b.v);
+            lx1a += U;
+            lx2a += P * a.d;
+            lx2b += P * b.d;
+            if (di != 0) {
+                face(di, a, b);
+                P = cr * (di > 0 ? -fb1 : 1.0 - fb1);
+                U = cr * (a.v + b.v);
+                lx2a += P * a.d;
+                lx2b += P * b.d;
             }
-            lx1b += cr * dPr1 * U;
-            lx1a -= cr * dPr0 * U;
-            lx2b += cr * Pr * V;
-            lx2a += cr * Pr * W;
+            lx1b -= U;
         }
-        double Pt = 0.0, dPt1 = 0.0, dPt0 = 0.0;
-        for (int l = 0; l < 3; ++l) {
-            Pt += S1t[l] - S0t[l];
-            dPt1 += dS1t[l];
-            dPt0 += dS0t[l];
-            int row = j0 - 1 + l;
-            if (row < 0 || row > g.nth - 1) continue;
-            double U = 0.0, V = 0.0, W = 0.0;
-            for (int k = 0; k < 4; ++k) {
-                double L = A.lamJ[1][(size_t)row * A.ld + (i0 - 1 + k + NG)];
-                U += L * (S1r[k] + S0r[k]);
-                V += L * dS1r[k];
-                W += L * dS0r[k];
+        {   // J^theta: columns of the start and of the end at a theta face's row
+            const double *L = A.lamJ[1];
+            auto face = [&](int l, Pair2 &a, Pair2 &b) {
+                const double *s0 = L + (w0 + (int64_t)l * ld), *s1 = s0 + di;
+                a = pair_at(__ldg(s0), __ldg(s0 + 1), fa1);
+                b = pair_at(__ldg(s1), __ldg(s1 + 1), fb1);
+            };
+            Pair2 a, b;
+            face(0, a, b);
+            double P = cr * (fa2 - (dj == 0 ? fb2 : (dj > 0 ? 1.0 : 0.0))), U = cr * (a.v + b.v);
+            lx2a += U;
+            lx1a += P * a.d;
+            lx1b += P * b.d;
+            if (dj != 0) {  // (the end's row j1: the extra face lies in the grid)
+                face(dj, a, b);
+                P = cr * (dj > 0 ? -fb2 : 1.0 - fb2);
+                U = cr * (a.v + b.v);
+                lx1a += P * a.d;
+                lx1b += P * b.d;
             }
-            lx1b += cr * Pt * V;
-            lx1a += cr * Pt * W;
-            lx2b += cr * dPt1 * U;
-            lx2a -= cr * dPt0 * U;
+            lx2b -= U;
         }
-        double At[4], Bt[4], LC[4] = {0, 0, 0, 0}, LD[4] = {0, 0, 0, 0};
-        for (int l = 0; l < 4; ++l) {
-            At[l] = c3 * S1t[l] + c6 * S0t[l];
-            Bt[l] = c6 * S1t[l] + c3 * S0t[l];
+        {   // J^phi: the four corner sets
+            const double *L = A.lamJ[2];
+            auto corners = [&](const double *q, double f1, double f2, double &I, double &I1, double &I2) {
+                Pair2 a = pair_at(__ldg(q), __ldg(q + 1), f1), b = pair_at(__ldg(q + ld), __ldg(q + ld + 1), f1);
+                I2 = b.v - a.v;
+                I = fma(f2, I2, a.v);
+                I1 = fma(f2, b.d - a.d, a.d);
+            };
+            double I00, R00, T00, I01, R01, T01, I10, R10, T10, I11, R11, T11;
+            corners(L + w0, fa1, fa2, I00, R00, T00);
+            corners(L + (w0 + (int64_t)dj * ld), fa1, fb2, I01, R01, T01);
+            corners(L + (w0 + di), fb1, fa2, I10, R10, T10);
+            corners(L + w1, fb1, fb2, I11, R11, T11);
+            const double c3 = 1.0 / 3.0, c6 = 1.0 / 6.0;
+            double p3 = cp * c3, p6 = cp * c6;
+            ldphi += cq * fma(c3, I11 + I00, c6 * (I10 + I01));
+            lx1a = fma(p3, R00, fma(p6, R01, lx1a));
+            lx1b = fma(p3, R11, fma(p6, R10, lx1b));
+            lx2a = fma(p3, T00, fma(p6, T10, lx2a));
+            lx2b = fma(p3, T11, fma(p6, T01, lx2b));
         }
-        for (int k = 0; k < 4; ++k) {
-            const double Ck = c3 * S1r[k] + c6 * S0r[k], Dk = c6 * S1r[k] + c3 * S0r[k];
-            double LA = 0.0, LB = 0.0;
-            for (int l = 0; l < 4; ++l) {
-                int row = j0 - 1 + l;
-                if (row < 0 || row > g.nth) continue;
-                double L = A.lamJ[2][(size_t)row * A.ld + (i0 - 1 + k + NG)];
-                LA += L * At[l];
-                LB += L * Bt[l];
-                LC[l] += L * Ck;
-                LD[l] += L * Dk;
-            }
-            ldphi += cq * (S1r[k] * LA + S0r[k] * LB);
-            lx1b += cp * dS1r[k] * LA;
-            lx1a += cp * dS0r[k] * LB;
-        }
-        for (int l = 0; l < 4; ++l) {
-            lx2b += cp * dS1t[l] * LC[l];
-            lx2a += cp * dS0t[l] * LD[l];
-        }
+        if (zero64(fa1)) lx1a = 0.0;
+        if (zero64(fa2)) lx2a = 0.0;
+        if (zero64(fb1)) lx1b = 0.0;
+        if (zero64(fb2)) lx2b = 0.0;
     }
     // end point: logical -> (r, theta) after reflection, then the reflection
-    l1[0] += lx1b / (y1[0] * g.dx1);
-    l1[1] += lx2b / g.dth;
+    l1[0] = fma(lx1b, rcp_t(y1[0]) * g.idx1, l1[0]);
+    l1[1] = fma(lx2b, g.idth, l1[1]);
     l1[1] *= refl;
     l1[3] *= refl;
     const double hh = 0.5 * dt;
@@ -701,8 +687,9 @@ __global__ void __launch_bounds__(128) particle_adjoint(PAdjArgs A)
         for (int k = 0; k < 5; ++k) l0[k] = ly0[k] + v0[k];
     }
     // start point: deposit's start-weight derivatives
-    l0[0] += lx1a / (r * g.dx1);
-    l0[1] += lx2a / g.dth;
+    const double ir1 = rcp_t(r) * g.idx1;  // d x1 / d r
+    l0[0] = fma(lx1a, ir1, l0[0]);
+    l0[1] = fma(lx2a, g.idth, l0[1]);
     // Boris: y0 = (r, th, u'(r, th, u, E))
     out[0] = l0[0];
     out[1] = l0[1];
@@ -710,12 +697,18 @@ __global__ void __launch_bounds__(128) particle_adjoint(PAdjArgs A)
         // fields at x^n and their logical derivatives
         St S[6];
         double E[6], dE1[6], dE2[6];
-        stencil(g, x1a, x2a, true, false, 1.0, S[0]);   // D^r
-        stencil(g, x1a, x2a, false, true, -1.0, S[1]);  // D^th (odd across the axis)
-        stencil(g, x1a, x2a, false, false, 1.0, S[2]);  // D^ph
-        stencil(g, x1a, x2a, false, true, 1.0, S[3]);   // B^r
-        stencil(g, x1a, x2a, true, false, 1.0, S[4]);   // B^th
-        stencil(g, x1a, x2a, true, true, 1.0, S[5]);    // B^ph
+        int ih, jh;
+        double fh, gh;
+        half_node(i0, fa1, ih, fh);
+        half_node(j0, fa2, jh, gh);
+        const bool m0 = jh < 0, m1 = jh + 1 > g.nth - 1;  // rows mirrored at the axis
+        const int h0 = m0 ? 0 : jh, h1 = m1 ? g.nth - 1 : jh + 1;
+        S[0] = {ih + NG, j0, j0 + 1, fh, fa2, false, false};  // D^r
+        S[1] = {i0 + NG, h0, h1, fa1, gh, m0, m1};            // D^th (odd across the axis)
+        S[2] = {i0 + NG, j0, j0 + 1, fa1, fa2, false, false};  // D^ph
+        S[3] = {i0 + NG, h0, h1, fa1, gh, false, false};      // B^r
+        S[4] = S[0];                                          // B^th
+        S[5] = {ih + NG, h0, h1, fh, gh, false, false};       // B^ph
         for (int c = 0; c < 6; ++c) gather_d(A.F[c], A.ld, S[c], E[c], dE1[c], dE2[c]);
         double zv[11] = {r, th, u[0], u[1], u[2], E[0], E[1], E[2], E[3], E[4], E[5]};
         double lb[11];
@@ -731,8 +724,8 @@ __global__ void __launch_bounds__(128) particle_adjoint(PAdjArgs A)
             lx1 += lE[c] * dE1[c];
             lx2 += lE[c] * dE2[c];
         }
-        out[0] += lx1 / (r * g.dx1);
-        out[1] += lx2 / g.dth;
+        out[0] = fma(lx1, ir1, out[0]);
+        out[1] = fma(lx2, g.idth, out[1]);
     } else {
         for (int k = 0; k < 3; ++k) out[2 + k] = l0[2 + k];
     }

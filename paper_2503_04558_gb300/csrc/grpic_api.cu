@@ -399,6 +399,7 @@ grpic_status grpic_init(grpic_metric metric, double spin, const grpic_grid *grid
     g.dth = M_PI / grid->n_theta;
     g.ln_rin = std::log(grid->r_in);
     g.idth = 1.0 / g.dth;
+    g.idx1 = 1.0 / g.dx1;
     gauss_legendre(NGL, ctx->gl_x, ctx->gl_w);
     ctx->slab = (size_t)(g.nth + 1) * g.ld_tab;
     int64_t ncell = (int64_t)g.nr * g.nth;

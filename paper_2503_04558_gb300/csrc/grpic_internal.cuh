@@ -40,7 +40,7 @@ constexpr int CELL_TERMS = 16;  // terms of the cell offset's series at most
 struct GridDev {
     int nr, nth, ld_tab;
     double a, r_in, r_out, dx1, dth, ln_rin;
-    double idth;  // 1 / dth
+    double idth, idx1;  // 1 / dth, 1 / dx1
     // FP64 contexts: where a particle's cell and its sin, cos come from without
     // the library's logarithm and sin / cos.  rcen: centre r_{i+1/2} of every
     // column (index i + NG) and its inverse; the offset in the cell is
@@ -267,6 +267,15 @@ __device__ __forceinline__ ColPos r_column_in(const GridDev &g, double r)
     if (c.i < 0) c = {0, 0.0};
     if (c.i > g.nr - 1) c = {g.nr - 1, 0x1.fffffffffffffp-1};
     return c;
+}
+
+// a lattice's bilinear stencil along one dimension: lower node and offset; the
+// half-integer lattice lies half a cell on
+__device__ __forceinline__ void half_node(int i, double f, int &ih, double &fh)
+{
+    const bool low = __double2hiint(f) < 0x3fe00000;  // f < 1/2
+    ih = low ? i - 1 : i;
+    fh = f + (low ? 0.5 : -0.5);
 }
 
 __device__ inline void set_status(int *st, int code) { atomicCAS(st, 0, code); }

@@ -152,6 +152,7 @@ extern "C" grpic_status grpic_sort_noalloc(const grpic_grid *grid, int32_t preci
     g.dx1 = std::log(grid->r_out / grid->r_in) / grid->n_r;
     g.dth = M_PI / grid->n_theta;
     g.idth = 1.0 / g.dth;
+    g.idx1 = 1.0 / g.dx1;
     g.ln_rin = std::log(grid->r_in);
     ctx.d_keys = sc->keys;
     ctx.d_perm = sc->perm;

@@ -253,15 +253,6 @@ __device__ __forceinline__ void vay(double a, double a2, const Pt64 &Bm, double 
     vay_step<double>(m, qm, dt, D, B, u);
 }
 
-// a lattice's bilinear stencil along one dimension: lower node and offset; the
-// half-integer lattice lies half a cell on
-__device__ __forceinline__ void half_node(int i, double f, int &ih, double &fh)
-{
-    const bool low = __double2hiint(f) < 0x3fe00000;  // f < 1/2
-    ih = low ? i - 1 : i;
-    fh = f + (low ? 0.5 : -0.5);
-}
-
 // a component from its four corners, along r on both rows, then along theta;
 // flip0, flip1: the rows are mirror rows of an odd component
 __device__ __forceinline__ double gather(const double *__restrict__ F, int64_t ld, int r0, int r1, int col, double f,
