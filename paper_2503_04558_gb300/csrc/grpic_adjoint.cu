@@ -746,108 +746,11 @@ __device__ __forceinline__ double tb(const FAdj &A, int slot, int i, int j)
     return A.tab[slot * A.slab + (size_t)j * A.ldt + (i + NG)];
 }
 
-// lamC (6 arrays at physical points) -> aux adjoints lamA[0..5] = H_r, H_th,
-// H_ph, E_r, E_th, E_ph (transpose of the circulations, Eqs. D-update, B-update)
-__global__ void circ_T(FAdj A, const double *const *lamC, double *const *lamA, double dth)
-{
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    int j = blockIdx.y * blockDim.y + threadIdx.y;
-    if (i > A.nr || j > A.nth) return;
-    const int nr = A.nr, nth = A.nth;
-    size_t q = (size_t)j * A.ld + (i + NG);
-    auto at = [&](double *L, int ii, int jj, double v) { atomicAdd(L + (size_t)jj * A.ld + (ii + NG), v); };
-    double drd = A.col1d[1 * A.ldt + i + NG], drp = A.col1d[0 * A.ldt + i + NG];
-    if (i <= nr - 1) {
-        double gv = lamC[0][q] * tb(A, T_INV_ADR, i, j);
-        if (j < nth) at(lamA[2], i, j, gv);
-        if (j > 0) at(lamA[2], i, j - 1, -gv);
-    }
-    if (j < nth) {
-        double gv = lamC[1][q] * tb(A, T_INV_ADT, i, j);
-        at(lamA[2], i - 1, j, gv);
-        at(lamA[2], i, j, -gv);
-        double gb = lamC[3][q] * tb(A, T_INV_ABR, i, j);
-        at(lamA[5], i, j + 1, -gb);
-        at(lamA[5], i, j, gb);
-    }
-    if (j > 0 && j < nth) {
-        double gv = lamC[2][q] * tb(A, T_INV_ADP, i, j);
-        at(lamA[1], i, j, gv * dth);
-        at(lamA[1], i - 1, j, -gv * dth);
-        at(lamA[0], i, j - 1, gv * drd);
-        at(lamA[0], i, j, -gv * drd);
-        if (i <= nr - 1) {
-            double gb = lamC[4][q] * tb(A, T_INV_ABT, i, j);
-            at(lamA[5], i, j, -gb);
-            at(lamA[5], i + 1, j, gb);
-        }
-    }
-    if (i <= nr - 1 && j < nth) {
-        double gb = lamC[5][q] * tb(A, T_INV_ABP, i, j);
-        at(lamA[4], i + 1, j, -gb * dth);
-        at(lamA[4], i, j, gb * dth);
-        at(lamA[3], i, j, -gb * drp);
-        at(lamA[3], i, j + 1, gb * drp);
-    }
-}
-
-// aux adjoints -> field adjoints (transpose of Eqs. auxH, auxE); one thread per
-// storage column/row, scatter with atomics
-__global__ void aux_T(FAdj A, const double *const *lamA, double *const *lamX)
-{
-    int col = blockIdx.x * blockDim.x + threadIdx.x;
-    int j = blockIdx.y * blockDim.y + threadIdx.y;
-    if (col < 1 || col > (int)A.ldt - 2 || j > A.nth) return;
-    int i = col - NG;
-    size_t q = (size_t)j * A.ld + col;
-    auto at = [&](double *L, int ii, int jj, double v) {
-        if (v != 0.0) atomicAdd(L + (size_t)jj * A.ld + (ii + NG), v);
-    };
-    double h;
-    // fields: 0 D^r, 1 D^th, 2 D^ph, 3 B^r, 4 B^th, 5 B^ph
-    if (j < A.nth) {
-        h = lamA[0][q];  // H_r
-        if (h != 0.0) {
-            at(lamX[3], i, j, tb(A, T_AGRR_BR, i, j) * h);
-            at(lamX[5], i, j, 0.5 * tb(A, T_AGRP_BP, i, j) * h);
-            at(lamX[5], i - 1, j, 0.5 * tb(A, T_AGRP_BP, i - 1, j) * h);
-        }
-        h = lamA[2][q];  // H_ph
-        if (h != 0.0) {
-            at(lamX[5], i, j, tb(A, T_AGPP_BP, i, j) * h);
-            at(lamX[3], i, j, 0.5 * tb(A, T_AGRP_BR, i, j) * h);
-            at(lamX[3], i + 1, j, 0.5 * tb(A, T_AGRP_BR, i + 1, j) * h);
-            at(lamX[1], i, j, -0.5 * tb(A, T_SGB_DT, i, j) * h);
-            at(lamX[1], i + 1, j, -0.5 * tb(A, T_SGB_DT, i + 1, j) * h);
-        }
-        h = lamA[4][q];  // E_th
-        if (h != 0.0) {
-            at(lamX[1], i, j, tb(A, T_AGTT_DT, i, j) * h);
-            at(lamX[5], i, j, -0.5 * tb(A, T_SGB_BP, i, j) * h);
-            at(lamX[5], i - 1, j, -0.5 * tb(A, T_SGB_BP, i - 1, j) * h);
-        }
-    }
-    h = lamA[1][q];  // H_th
-    if (h != 0.0) {
-        at(lamX[4], i, j, tb(A, T_AGTT_BT, i, j) * h);
-        at(lamX[2], i, j, 0.5 * tb(A, T_SGB_DP, i, j) * h);
-        at(lamX[2], i + 1, j, 0.5 * tb(A, T_SGB_DP, i + 1, j) * h);
-    }
-    h = lamA[3][q];  // E_r
-    if (h != 0.0) {
-        at(lamX[0], i, j, tb(A, T_AGRR_DR, i, j) * h);
-        at(lamX[2], i, j, 0.5 * tb(A, T_AGRP_DP, i, j) * h);
-        at(lamX[2], i + 1, j, 0.5 * tb(A, T_AGRP_DP, i + 1, j) * h);
-    }
-    h = lamA[5][q];  // E_ph
-    if (h != 0.0) {
-        at(lamX[2], i, j, tb(A, T_AGPP_DP, i, j) * h);
-        at(lamX[0], i, j, 0.5 * tb(A, T_AGRP_DR, i, j) * h);
-        at(lamX[0], i - 1, j, 0.5 * tb(A, T_AGRP_DR, i - 1, j) * h);
-        at(lamX[4], i, j, 0.5 * tb(A, T_SGB_BT, i, j) * h);
-        at(lamX[4], i - 1, j, 0.5 * tb(A, T_SGB_BT, i - 1, j) * h);
-    }
-}
+// device pointers of up to six arrays, passed by value
+struct P6 {
+    double *p[6];
+    __host__ __device__ double *operator[](int k) const { return p[k]; }
+};
 
 __device__ __forceinline__ bool phys(int comp, int i, int j, int nr, int nth)
 {
@@ -857,68 +760,141 @@ __device__ __forceinline__ bool phys(int comp, int i, int j, int nr, int nth)
     return true;
 }
 
-// transpose of the boundary projection P of one stage (with damping when
-// damp != 0): mu[phys] = damp * (lam[phys] + lam of the guard copies of it);
-// axis D^ph, B^th rows and non-physical entries get 0
-__global__ void proj_T(FAdj A, const double *const *lam, double *const *mu, int damp)
+// The field update's transpose works on mu_k, the adjoint of stage k's value before
+// its boundary copies.  A stage's mu gives the adjoints h of the auxiliary
+// fields (transpose of the circulations), these the previous iterate's adjoint
+// (transpose of the auxiliary fields), and the guard copies' transpose the
+// previous mu: two launches a stage, every entry gathered by its own thread (the
+// scatter with atomics took 8 launches and 12 clears).  The sums over the stages
+// that the rest needs follow from M = sum_k mu_k and mu_0.
+
+// mu (zero where a component is not updated) -> scale * h: H_r, H_th, H_ph, E_r,
+// E_th, E_ph (transpose of Eqs. D-update, B-update), every column and row
+__global__ void __launch_bounds__(256) stage_h(FAdj A, P6 mu, P6 h, double scale, double dth)
 {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    int j = blockIdx.y * blockDim.y + threadIdx.y;
-    if (i > A.nr || j > A.nth) return;
-    for (int comp = 0; comp < 6; ++comp) {
-        size_t row = (size_t)j * A.ld;
-        double v = 0.0;
-        if (phys(comp, i, j, A.nr, A.nth) && !((comp == 2 || comp == 4) && (j == 0 || j == A.nth))) {
-            bool half_r = (comp == 0 || comp == 4 || comp == 5);
-            int last = half_r ? A.nr - 1 : A.nr;
-            v = lam[comp][row + i + NG];
-            if (i == 0) v += lam[comp][row + 0] + lam[comp][row + 1];
-            if (i == last)
-                for (int c = last + 1 + NG; c < A.nr + 2 * NG; ++c) v += lam[comp][row + c];
-            if (damp) v *= A.col1d[(half_r ? 3 : 2) * A.ldt + i + NG];
-        }
-        mu[comp][row + i + NG] = v;
-        if (i == 0) { mu[comp][row + 0] = 0.0; mu[comp][row + 1] = 0.0; }
-        if (i == A.nr)
-            for (int c = A.nr + 1 + NG; c < A.nr + 2 * NG; ++c) mu[comp][row + c] = 0.0;
+    const int c = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y;
+    if (c >= (int)A.ldt || j > A.nth) return;
+    const int i = c - NG;
+    const int inv[6] = {T_INV_ADR, T_INV_ADT, T_INV_ADP, T_INV_ABR, T_INV_ABT, T_INV_ABP};
+    auto g = [&](int k, int ii, int jj) {
+        if (ii < 0 || ii > A.nr || jj < 0 || jj > A.nth) return 0.0;
+        return __ldg(mu[k] + (size_t)jj * A.ld + (ii + NG)) * tb(A, inv[k], ii, jj);
+    };
+    const double drp = A.col1d[c], drd = A.col1d[A.ldt + c];
+    const size_t q = (size_t)j * A.ld + c;
+    const double g1 = g(1, i, j), g2 = g(2, i, j), g5 = g(5, i, j);
+    h[0][q] = scale * (g(2, i, j + 1) - g2) * drd;
+    h[1][q] = scale * (g2 - g(2, i + 1, j)) * dth;
+    h[2][q] = scale * ((j < A.nth ? g(0, i, j) : 0.0) - g(0, i, j + 1) + g(1, i + 1, j) - g1);
+    h[3][q] = scale * (g(5, i, j - 1) - g5) * drp;
+    h[4][q] = scale * (g5 - g(5, i - 1, j)) * dth;
+    h[5][q] = scale * (g(3, i, j) - g(3, i, j - 1) + g(4, i - 1, j) - g(4, i, j));
+}
+
+// component k of the iterate's adjoint at (column c, row j) from h (transpose of
+// Eqs. auxH, auxE); zero beyond the columns
+__device__ __forceinline__ double from_h(const FAdj &A, const P6 &h, int k, int c, int j)
+{
+    if (c < 0 || c >= (int)A.ldt) return 0.0;
+    const int i = c - NG;
+    const size_t q = (size_t)j * A.ld + c;
+    const bool l = c > 0, r = c + 1 < (int)A.ldt;
+    auto pair = [&](int n, bool right) {
+        const double *x = h[n] + q;
+        return __ldg(x) + (right ? (r ? __ldg(x + 1) : 0.0) : (l ? __ldg(x - 1) : 0.0));
+    };
+    switch (k) {
+    case 0: return tb(A, T_AGRR_DR, i, j) * __ldg(h[3] + q) + 0.5 * tb(A, T_AGRP_DR, i, j) * pair(5, true);
+    case 1: return tb(A, T_AGTT_DT, i, j) * __ldg(h[4] + q) - 0.5 * tb(A, T_SGB_DT, i, j) * pair(2, false);
+    case 2:
+        return tb(A, T_AGPP_DP, i, j) * __ldg(h[5] + q) + 0.5 * (tb(A, T_SGB_DP, i, j) * pair(1, false) +
+                                                                  tb(A, T_AGRP_DP, i, j) * pair(3, false));
+    case 3: return tb(A, T_AGRR_BR, i, j) * __ldg(h[0] + q) + 0.5 * tb(A, T_AGRP_BR, i, j) * pair(2, false);
+    case 4: return tb(A, T_AGTT_BT, i, j) * __ldg(h[1] + q) + 0.5 * tb(A, T_SGB_BT, i, j) * pair(5, true);
+    default:
+        return tb(A, T_AGPP_BP, i, j) * __ldg(h[2] + q) + 0.5 * (tb(A, T_AGRP_BP, i, j) * pair(0, true) -
+                                                                  tb(A, T_SGB_BP, i, j) * pair(4, true));
     }
 }
 
-// entries a field update never writes (rows past the last half-theta row,
-// columns past the last guard) keep their value: the identity
-__global__ void passthru(FAdj A, const double *const *lamIn, double *const *lamOut)
+// the boundary copies' transpose of X(column): the physical columns' values plus
+// those of their guard copies, zero in the guards and on the axis (D^ph, B^th)
+template <typename XF>
+__device__ __forceinline__ void put_mu(const FAdj &A, int k, int i, int j, const XF &X, double damp, P6 mu, P6 M,
+                                       bool add)
 {
-    int c = blockIdx.x * blockDim.x + threadIdx.x;
-    int j = blockIdx.y * blockDim.y + threadIdx.y;
+    const bool hr = (k == 0 || k == 4 || k == 5);
+    const size_t row = (size_t)j * A.ld;
+    double v = 0.0;
+    if (phys(k, i, j, A.nr, A.nth) && !((k == 2 || k == 4) && (j == 0 || j == A.nth))) {
+        const int last = hr ? A.nr - 1 : A.nr;
+        v = X(i + NG);
+        if (i == 0) v += X(0) + X(1);
+        if (i == last)
+            for (int c = last + 1 + NG; c < A.nr + 2 * NG; ++c) v += X(c);
+        v *= damp;
+    }
+    const size_t q = row + i + NG;
+    mu[k][q] = v;
+    M[k][q] = add ? M[k][q] + v : v;
+    for (int c = 0; c < NG && i == 0; ++c) mu[k][row + c] = M[k][row + c] = 0.0;
+    for (int c = A.nr + 1 + NG; c < A.nr + 2 * NG && i == A.nr; ++c) mu[k][row + c] = M[k][row + c] = 0.0;
+}
+
+// mu, M <- the projection's transpose of lam (the last stage's, damped)
+__global__ void __launch_bounds__(256) stage_first(FAdj A, P6 lam, P6 mu, P6 M, int damp)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y;
+    if (i > A.nr || j > A.nth) return;
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+        const double *L = lam[k] + (size_t)j * A.ld;
+        const double f = damp ? A.col1d[((k == 0 || k == 4 || k == 5) ? 3 : 2) * A.ldt + i + NG] : 1.0;
+        put_mu(A, k, i, j, [&](int c) { return __ldg(L + c); }, f, mu, M, false);
+    }
+}
+
+// mu <- the previous stage's from h; M += mu
+__global__ void __launch_bounds__(256) stage_mu(FAdj A, P6 h, P6 mu, P6 M)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y;
+    if (i > A.nr || j > A.nth) return;
+#pragma unroll
+    for (int k = 0; k < 6; ++k)
+        put_mu(A, k, i, j, [&](int c) { return from_h(A, h, k, c, j); }, 1.0, mu, M, true);
+}
+
+// after the stages: lam_out <- M (the identity for entries that an update never
+// writes: rows past the last half-theta row, columns past the last guard),
+// lam_J <- -dt M / A, mu <- dt (alpha_s (M - mu_0) + mu_0) = the adjoint of C(X^n)
+__global__ void __launch_bounds__(256) stages_close(FAdj A, P6 lam, P6 mu, P6 M, P6 out, P6 lamJ, double dt, double as)
+{
+    const int c = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y;
     if (c >= A.ld || j > A.nth) return;
-    size_t q = (size_t)j * A.ld + c;
-    for (int comp = 0; comp < 6; ++comp) {
-        bool half_t = (comp == 1 || comp == 3 || comp == 5);
-        bool written = c < A.nr + 2 * NG && j <= (half_t ? A.nth - 1 : A.nth);
-        if (!written) lamOut[comp][q] += lamIn[comp][q];
+    const int i = c - NG, inv[3] = {T_INV_ADR, T_INV_ADT, T_INV_ADP};
+    const size_t q = (size_t)j * A.ld + c;
+    const bool in = c < (int)A.ldt;
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+        const bool ht = (k == 1 || k == 3 || k == 5);
+        const bool written = in && j <= (ht ? A.nth - 1 : A.nth);
+        const double m = in ? M[k][q] : 0.0;
+        out[k][q] = written ? m : lam[k][q];
+        if (in) {
+            const double m0 = mu[k][q];
+            mu[k][q] = dt * (as * (m - m0) + m0);
+        }
+        if (k < 3) lamJ[k][q] = in && i >= 0 && i <= A.nr ? -dt * m * tb(A, inv[k], i, j) : 0.0;
     }
 }
 
-// y[k] += s * x[k] over n elements of 6 arrays
-__global__ void axpy6(double *const *y, const double *const *x, double s, size_t n)
+// out += the iterate's adjoint from h, entry by entry
+__global__ void __launch_bounds__(256) add_from_h(FAdj A, P6 h, P6 out)
 {
-    size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= n) return;
-    for (int k = 0; k < 6; ++k) y[k][e] += s * x[k][e];
-}
-
-// lamJ[k] (J A adjoint) += s * invA^D_k * mu_D[k] at physical D points
-__global__ void jadj(FAdj A, const double *const *mu, double *const *lamJ, double s)
-{
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    int j = blockIdx.y * blockDim.y + threadIdx.y;
-    if (i > A.nr || j > A.nth) return;
-    const int inv[3] = {T_INV_ADR, T_INV_ADT, T_INV_ADP};
-    for (int k = 0; k < 3; ++k)
-        if (phys(k, i, j, A.nr, A.nth)) {
-            size_t q = (size_t)j * A.ld + i + NG;
-            lamJ[k][q] += s * tb(A, inv[k], i, j) * mu[k][q];
-        }
+    const int c = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y;
+    if (c >= (int)A.ldt || j > A.nth) return;
+#pragma unroll
+    for (int k = 0; k < 6; ++k) out[k][(size_t)j * A.ld + c] += from_h(A, h, k, c, j);
 }
 
 // ---- objective ------------------------------------------------------------
@@ -928,7 +904,7 @@ __device__ __forceinline__ double fx(const double *F, int64_t ld, int i, int j) 
 struct Ring {
     double Eth, Hph, Eph, Hth;
 };
-__device__ Ring ring_vals(FAdj A, const double *const *F, int iH, int j)
+__device__ Ring ring_vals(FAdj A, P6 F, int iH, int j)
 {
     auto Hph = [&](int i, int jj) {
         return tb(A, T_AGPP_BP, i, jj) * fx(F[5], A.ld, i, jj) +
@@ -957,7 +933,7 @@ __device__ Ring ring_vals(FAdj A, const double *const *F, int iH, int j)
 }
 
 // flux at the ring (one block reduction) accumulated into *out with weight w
-__global__ void flux_kernel(FAdj A, const double *const *F, int iH, double dth, double w, double *out)
+__global__ void flux_kernel(FAdj A, P6 F, int iH, double dth, double w, double *out)
 {
     __shared__ double red[256];
     double s = 0.0;
@@ -975,7 +951,7 @@ __global__ void flux_kernel(FAdj A, const double *const *F, int iH, double dth, 
 }
 
 // seed: aux adjoints of w * flux (then aux_T maps them to the fields)
-__global__ void flux_seed(FAdj A, const double *const *F, int iH, double dth, double w, double *const *lamA)
+__global__ void flux_seed(FAdj A, P6 F, int iH, double dth, double w, P6 lamA)
 {
     int j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= A.nth) return;
@@ -1008,7 +984,7 @@ __device__ __forceinline__ VD operator*(double c, VD x) { return {c * x.v, c * x
 struct DAux {
     FAdj A;
     const double *dtab;
-    const double *const *X;
+    P6 X;
     __device__ VD p(int slot, int comp, int i, int j) const
     {
         size_t q = slot * A.slab + (size_t)j * A.ldt + (i + NG);
@@ -1064,8 +1040,8 @@ __device__ __forceinline__ void block_add(double v, double *out)
 
 // *out += sum over points of w . dC/da (X): C the circulation of one stage
 // (Eqs. D-update, B-update divided by the face areas), w adjoint-shaped
-__global__ void __launch_bounds__(256) dcirc_dot(FAdj A, const double *dtab, const double *const *X,
-                                                 const double *const *w, double dth, double *out)
+__global__ void __launch_bounds__(256) dcirc_dot(FAdj A, const double *dtab, P6 X, P6 w, double scale, double dth,
+                                                 double *out)
 {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     int j = blockIdx.y * blockDim.y + threadIdx.y;
@@ -1096,13 +1072,13 @@ __global__ void __launch_bounds__(256) dcirc_dot(FAdj A, const double *dtab, con
             acc += term(5, T_INV_ABP,
                         -1.0 * (dth * (X_.Eth(i + 1, j) - X_.Eth(i, j)) + drp * (X_.Er(i, j) - X_.Er(i, j + 1))));
     }
-    block_add(acc, out);
+    block_add(scale * acc, out);
 }
 
 // *out += sj * sum over the D points a stage writes of w . d(invA)/da J A
 // (the current term of Eq. fld-predictor / fld-corrector)
-__global__ void __launch_bounds__(256) jinv_dot(FAdj A, const double *dtab, const double *const *w,
-                                                const double *const *J, double sj, double *out)
+__global__ void __launch_bounds__(256) jinv_dot(FAdj A, const double *dtab, P6 w,
+                                                P6 J, double sj, double *out)
 {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     int j = blockIdx.y * blockDim.y + threadIdx.y;
@@ -1117,7 +1093,7 @@ __global__ void __launch_bounds__(256) jinv_dot(FAdj A, const double *dtab, cons
 }
 
 // *out += w * d(flux)/da at fixed fields F (the ring values of the objective)
-__global__ void __launch_bounds__(256) flux_da(FAdj A, const double *dtab, const double *const *F, int iH, double dth,
+__global__ void __launch_bounds__(256) flux_da(FAdj A, const double *dtab, P6 F, int iH, double dth,
                                                double w, double *out)
 {
     double acc = 0.0;
@@ -1155,21 +1131,11 @@ using namespace grpic;
 
 namespace {
 
-struct Bufs {
-    size_t fn;      // elements of one field array
-    int64_t np;     // particles
-};
-
-// device pointer arrays for kernels taking "double *const *" (6 entries)
-struct PtrSet {
-    double **d;  // device array of 6 (or 3) pointers
-};
-
-cudaError_t upload_ptrs(double *const *h, int n, double ***d, cudaStream_t s)
+P6 six(double *const *h, int n = 6)
 {
-    cudaError_t e = cudaMalloc(d, sizeof(double *) * n);
-    if (e != cudaSuccess) return e;
-    return cudaMemcpyAsync(*d, h, sizeof(double *) * n, cudaMemcpyHostToDevice, s);
+    P6 q;
+    for (int k = 0; k < 6; ++k) q.p[k] = k < n ? h[k] : nullptr;
+    return q;
 }
 
 }  // namespace
@@ -1186,89 +1152,57 @@ extern "C" grpic_status grpic_horizon_flux(grpic_ctx *ctx, const grpic_fields *f
         hp[k] = (double *)f->D[k];
         hp[3 + k] = (double *)f->B[k];
     }
-    double **dp = nullptr;
-    if (upload_ptrs(hp, 6, &dp, s) != cudaSuccess) return GRPIC_ENOMEM;
     FAdj A{ctx->g.nr, ctx->g.nth, f->ld, ctx->g.ld_tab, ctx->slab, ctx->tab, ctx->col1d};
-    cudaMemsetAsync(out, 0, sizeof(double), s);
-    flux_kernel<<<1, 256, 0, s>>>(A, dp, i_horizon, ctx->g.dth, 1.0, out);
+    double *dev = (double *)((char *)ctx->d_status + 48);  // behind the status word and the charges
+    cudaMemsetAsync(dev, 0, sizeof(double), s);
+    flux_kernel<<<1, 256, 0, s>>>(A, six(hp), i_horizon, ctx->g.dth, 1.0, dev);
     cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaMemcpyAsync(out, dev, sizeof(double), cudaMemcpyDeviceToHost, s);
     cudaStreamSynchronize(s);
-    cudaFree(dp);
     return e == cudaSuccess ? GRPIC_OK : GRPIC_ECUDA;
 }
 
 // What the spin derivative of one field update needs: the derivative
 // tables, the update's input fields Xn, its currents J and every stage's
-// output Y[k] (device pointer arrays), and the scalar it accumulates into.
+// output Y[6 k ..], and the scalar it accumulates into.
 struct SpinField {
     const double *dtab;
-    double **Xn;   // 6
-    double **J;    // 3
-    double **Y;    // (n_field_iter + 1) * 6
+    P6 Xn, J;
+    double *const *Y;
     double *La;
 };
 
-// Transpose of one field update: lam (adjoint of F^{n+1}, in f_lam->D/B) ->
-// adjoint of F^n (out->D/B) and of the integrated currents J A (out->J).
+// Transpose of one field update: lam (adjoint of F^{n+1}) -> out, the adjoint of
+// F^n, and lamJ, of the integrated currents J A.  work: mu[6], M[6], h[6].
 // With sp, also adds the update's a-derivative contracted with the stage
 // adjoints to sp->La: every stage's pre-projection value
 //   dt (c_k C(Xn) + beta_s C(Y_{k-1})) - dt invA J   (c_0 = 1, c_k = alpha_s)
 // depends on a through the tables of C and invA.
-static grpic_status field_adjoint(grpic_ctx *ctx, double **lamIn, double **lamOut, double **lamJ, double **work,
-                                  int64_t ld, cudaStream_t s, double ***dptrs, const SpinField *sp = nullptr)
+static grpic_status field_adjoint(grpic_ctx *ctx, P6 lam, P6 out, P6 lamJ, double *const *work, int64_t ld,
+                                  cudaStream_t s, const SpinField *sp = nullptr)
 {
-    // work: mu[6], lamCn[6], lamPrev[6], aux[6]  (24 arrays); dptrs: device copies
     const int N = ctx->prm.n_field_iter;
-    const double dt = ctx->prm.dt, bs = ctx->prm.beta_field, as = 1.0 - bs;
-    size_t fn = (size_t)(ctx->g.nth + 1) * ld;
+    const double dt = ctx->prm.dt, bs = ctx->prm.beta_field, as = 1.0 - bs, dth = ctx->g.dth;
     FAdj A{ctx->g.nr, ctx->g.nth, ld, ctx->g.ld_tab, ctx->slab, ctx->tab, ctx->col1d};
-    dim3 blk(64, 4), grd((ctx->g.nr + 1 + 63) / 64, (ctx->g.nth + 1 + 3) / 4);
-    dim3 gfull((ctx->g.ld_tab + 63) / 64, (ctx->g.nth + 1 + 3) / 4);
-    unsigned nb = (unsigned)((fn + 255) / 256);
-    double **d_in = dptrs[0], **d_out = dptrs[1], **d_J = dptrs[2], **d_mu = dptrs[3], **d_lcn = dptrs[4],
-           **d_prev = dptrs[5], **d_aux = dptrs[6], **d_cur = dptrs[7];
-    double **mu = work, **lcn = work + 6, **prev = work + 12, **aux = work + 18;
-    for (int k = 0; k < 6; ++k) {
-        cudaMemsetAsync(lamOut[k], 0, fn * sizeof(double), s);
-        cudaMemsetAsync(lcn[k], 0, fn * sizeof(double), s);
-        cudaMemsetAsync(mu[k], 0, fn * sizeof(double), s);
+    const dim3 blk(64, 4), rows((ctx->g.nth + 1 + 3) / 4);
+    const dim3 gphys((ctx->g.nr + 1 + 63) / 64, rows.x), gcol((ctx->g.ld_tab + 63) / 64, rows.x),
+        gld((unsigned)((ld + 63) / 64), rows.x);
+    const P6 mu = six(work), M = six(work + 6), h = six(work + 12);
+    stage_first<<<gphys, blk, 0, s>>>(A, lam, mu, M, 1);
+    for (int k = N; k > 0; --k) {
+        if (sp)  // dt beta_s mu_k . dC/da (Y_{k-1})
+            dcirc_dot<<<gphys, blk, 0, s>>>(A, sp->dtab, six(sp->Y + (k - 1) * 6), mu, dt * bs, dth, sp->La);
+        stage_h<<<gcol, blk, 0, s>>>(A, mu, h, dt * bs, dth);
+        stage_mu<<<gphys, blk, 0, s>>>(A, h, mu, M);
     }
-    for (int k = 0; k < 3; ++k) cudaMemsetAsync(lamJ[k], 0, fn * sizeof(double), s);
-    dim3 gld((unsigned)((ld + 63) / 64), (ctx->g.nth + 1 + 3) / 4);
-    passthru<<<gld, blk, 0, s>>>(A, d_in, d_out);
-    // current adjoint of the stage output: starts at lamIn
-    cudaMemcpyAsync(d_cur, d_in, sizeof(double *) * 6, cudaMemcpyDeviceToDevice, s);
-    for (int k = N; k >= 0; --k) {
-        // mu = P_k^T lam_k (damping in the last stage)
-        proj_T<<<grd, blk, 0, s>>>(A, d_cur, d_mu, (k == N && N > 0) ? 1 : 0);
-        // lam X^n (physical part) += mu; lam Cn += dt * (k==0 ? 1 : alpha) * mu; lam J -= dt * invA * mu
-        axpy6<<<nb, 256, 0, s>>>(d_out, d_mu, 1.0, fn);
-        axpy6<<<nb, 256, 0, s>>>(d_lcn, d_mu, dt * (k == 0 ? 1.0 : as), fn);
-        jadj<<<grd, blk, 0, s>>>(A, d_mu, d_J, -dt);
-        if (sp)  // the current term: -dt mu_k . d(invA)/da J
-            jinv_dot<<<grd, blk, 0, s>>>(A, sp->dtab, d_mu, sp->J, -dt, sp->La);
-        if (k > 0) {
-            // lam of the previous iterate = C^T (dt beta mu)
-            for (int c = 0; c < 6; ++c) {
-                cudaMemsetAsync(aux[c], 0, fn * sizeof(double), s);
-                cudaMemsetAsync(prev[c], 0, fn * sizeof(double), s);
-            }
-            // scale mu by dt*beta in place
-            axpy6<<<nb, 256, 0, s>>>(d_mu, d_mu, dt * bs - 1.0, fn);
-            if (sp)  // dt beta_s mu_k . dC/da (Y_{k-1})
-                dcirc_dot<<<grd, blk, 0, s>>>(A, sp->dtab, sp->Y + (k - 1) * 6, d_mu, ctx->g.dth, sp->La);
-            circ_T<<<grd, blk, 0, s>>>(A, d_mu, d_aux, ctx->g.dth);
-            aux_T<<<gfull, blk, 0, s>>>(A, d_aux, d_prev);
-            cudaMemcpyAsync(d_cur, d_prev, sizeof(double *) * 6, cudaMemcpyDeviceToDevice, s);
-        }
-    }
-    // (sum_k dt c_k mu_k) . dC/da (X^n)
-    if (sp) dcirc_dot<<<grd, blk, 0, s>>>(A, sp->dtab, sp->Xn, d_lcn, ctx->g.dth, sp->La);
-    // lam X^n += C^T lam Cn
-    for (int c = 0; c < 6; ++c) cudaMemsetAsync(aux[c], 0, fn * sizeof(double), s);
-    circ_T<<<grd, blk, 0, s>>>(A, d_lcn, d_aux, ctx->g.dth);
-    aux_T<<<gfull, blk, 0, s>>>(A, d_aux, d_out);
-    (void)lamIn;
+    if (sp)  // the currents' term: -dt M . d(invA)/da J
+        jinv_dot<<<gphys, blk, 0, s>>>(A, sp->dtab, M, sp->J, -dt, sp->La);
+    stages_close<<<gld, blk, 0, s>>>(A, lam, mu, M, out, lamJ, dt, as);
+    if (sp)  // (sum_k dt c_k mu_k) . dC/da (X^n)
+        dcirc_dot<<<gphys, blk, 0, s>>>(A, sp->dtab, sp->Xn, mu, 1.0, dth, sp->La);
+    // lam X^n += C^T lam C(X^n)
+    stage_h<<<gcol, blk, 0, s>>>(A, mu, h, 1.0, dth);
+    add_from_h<<<gcol, blk, 0, s>>>(A, h, out);
     return cudaGetLastError() == cudaSuccess ? GRPIC_OK : GRPIC_ECUDA;
 }
 
@@ -1281,10 +1215,10 @@ extern "C" grpic_status grpic_adjoint_field_step(grpic_ctx *ctx, const grpic_fie
     cudaStream_t s = (cudaStream_t)stream;
     int64_t ld = lam_in->ld;
     size_t fn = (size_t)(ctx->g.nth + 1) * ld;
-    std::vector<double *> work(24, nullptr);
-    for (auto &w : work)
-        if (cudaMalloc(&w, fn * sizeof(double)) != cudaSuccess) return GRPIC_ENOMEM;
-    double *in[6], *out[6], *J[3];
+    double *base = nullptr;
+    if (cudaMalloc(&base, 18 * fn * sizeof(double)) != cudaSuccess) return GRPIC_ENOMEM;
+    double *work[18], *in[6], *out[6], *J[3];
+    for (int k = 0; k < 18; ++k) work[k] = base + k * fn;
     for (int k = 0; k < 3; ++k) {
         in[k] = (double *)lam_in->D[k];
         in[3 + k] = (double *)lam_in->B[k];
@@ -1292,17 +1226,9 @@ extern "C" grpic_status grpic_adjoint_field_step(grpic_ctx *ctx, const grpic_fie
         out[3 + k] = (double *)lam_out->B[k];
         J[k] = (double *)lam_out->J[k];
     }
-    double **dp[8];
-    double *cur_dummy[6] = {0};
-    bool ok = upload_ptrs(in, 6, &dp[0], s) == cudaSuccess && upload_ptrs(out, 6, &dp[1], s) == cudaSuccess &&
-              upload_ptrs(J, 3, &dp[2], s) == cudaSuccess && upload_ptrs(&work[0], 6, &dp[3], s) == cudaSuccess &&
-              upload_ptrs(&work[6], 6, &dp[4], s) == cudaSuccess && upload_ptrs(&work[12], 6, &dp[5], s) == cudaSuccess &&
-              upload_ptrs(&work[18], 6, &dp[6], s) == cudaSuccess && upload_ptrs(cur_dummy, 6, &dp[7], s) == cudaSuccess;
-    grpic_status st = ok ? field_adjoint(ctx, in, out, J, work.data(), ld, s, dp) : GRPIC_ENOMEM;
+    grpic_status st = field_adjoint(ctx, six(in), six(out), six(J, 3), work, ld, s);
     cudaStreamSynchronize(s);
-    for (int k = 0; k < 8; ++k)
-        if (ok) cudaFree(dp[k]);
-    for (auto w : work) cudaFree(w);
+    cudaFree(base);
     return st;
 }
 
@@ -1331,87 +1257,102 @@ extern "C" grpic_status grpic_adjoint_grad(grpic_ctx *ctx, const grpic_particles
     const size_t fn = (size_t)(ctx->g.nth + 1) * ld;
     const int ck = checkpoint_every;
     const int nseg = (nsteps + ck - 1) / ck;
-    std::vector<void *> allocs;
-    auto dalloc = [&](size_t bytes) -> void * {
-        void *q = nullptr;
-        if (cudaMalloc(&q, bytes > 0 ? bytes : 8) != cudaSuccess) return nullptr;
-        allocs.push_back(q);
-        return q;
-    };
-    auto cleanup = [&]() {
-        cudaStreamSynchronize(s);
-        for (void *q : allocs) cudaFree(q);
-    };
-    // states: checkpoints (nseg) and the current segment's states (ck + 1)
+    const int sl = std::min(ck, nsteps);  // steps of the longest segment
+    const int last0 = (nseg - 1) * ck;    // first step of the last segment
+    const bool spin = dL_da != nullptr;
+    const int NF = ctx->prm.n_field_iter, TW = tape_width(ctx->prm.n_push_iter);
+    const size_t ntab = ctx->slab * T_COUNT;
+    // states: checkpoints of every segment but the last (which is recorded during
+    // the forward pass), the current segment's states
     struct State {
         double *F[6];
         double *x[5];
         uint32_t *tag;
     };
-    auto new_state = [&](State &S) -> bool {
-        for (int k = 0; k < 6; ++k)
-            if (!(S.F[k] = (double *)dalloc(fn * sizeof(double)))) return false;
-        for (int k = 0; k < 5; ++k)
-            if (!(S.x[k] = (double *)dalloc(np * sizeof(double)))) return false;
-        return (S.tag = (uint32_t *)dalloc(np * sizeof(uint32_t))) != nullptr;
+    std::vector<State> cks(want ? nseg - 1 : 0), seg(want ? sl + 1 : 0);
+    State W;  // working particles / fields of the forward runs
+    double *Jw[3], *Ldev, *lamFa[6], *lamFb[6], *lamJ[3], *lamP[5], *lamP2[5], *aux[6], *tape = nullptr;
+    std::vector<double *> work(want ? 18 : 0, nullptr);
+    // spin derivative: derivative tables (and those of a +- h), per-particle parts,
+    // the segment's currents and one update's stage outputs
+    double *dtab = nullptr, *tp = nullptr, *tm = nullptr, *c1 = nullptr, *Ladev = nullptr, *Lap = nullptr;
+    std::vector<double *> segJ(spin ? 3 * sl : 0, nullptr), Ystage(spin ? 6 * (NF + 1) : 0, nullptr);
+    // one block holds all of it: the first pass measures, the second places
+    char *base = nullptr;
+    size_t need = 0;
+    auto place = [&](size_t bytes) -> double * {
+        double *q = base ? (double *)(base + need) : nullptr;
+        need += (bytes + 255) & ~(size_t)255;
+        return q;
     };
-    std::vector<State> cks(want ? nseg : 0), seg(want ? ck + 1 : 0);
-    bool ok = true;
-    for (auto &S : cks) ok = ok && new_state(S);
-    for (auto &S : seg) ok = ok && new_state(S);
-    // working particles / fields for the forward runs
-    State W;
-    ok = ok && new_state(W);
-    double *Jw[3];
-    for (int k = 0; k < 3; ++k) ok = ok && (Jw[k] = (double *)dalloc(fn * sizeof(double)));
-    int64_t *cnt = (int64_t *)dalloc(sizeof(int64_t));
-    double *Ldev = (double *)dalloc(sizeof(double));
-    // adjoint arrays
-    double *lamF[6], *lamF2[6], *lamJ[3], *lamP[5], *lamP2[5], *aux[6];
-    for (int k = 0; k < 6; ++k) {
-        ok = ok && (lamF[k] = (double *)dalloc(fn * sizeof(double)));
-        ok = ok && (lamF2[k] = (double *)dalloc(fn * sizeof(double)));
-        ok = ok && (aux[k] = (double *)dalloc(fn * sizeof(double)));
+    auto layout = [&]() {
+        need = 0;
+        auto state = [&](State &S) {
+            for (int k = 0; k < 6; ++k) S.F[k] = place(fn * sizeof(double));
+            for (int k = 0; k < 5; ++k) S.x[k] = place(np * sizeof(double));
+            S.tag = (uint32_t *)place(np * sizeof(uint32_t));
+        };
+        for (auto &S : cks) state(S);
+        for (auto &S : seg) state(S);
+        state(W);
+        for (int k = 0; k < 3; ++k) Jw[k] = place(fn * sizeof(double));
+        Ldev = place(sizeof(double));
+        if (!want) return;
+        for (int k = 0; k < 6; ++k) lamFa[k] = place(fn * sizeof(double));
+        for (int k = 0; k < 6; ++k) lamFb[k] = place(fn * sizeof(double));
+        double *a6 = place(6 * fn * sizeof(double));
+        for (int k = 0; k < 6; ++k) aux[k] = a6 + (base ? k * fn : 0);
+        for (int k = 0; k < 3; ++k) lamJ[k] = place(fn * sizeof(double));
+        for (int k = 0; k < 5; ++k) lamP[k] = place(np * sizeof(double));
+        for (int k = 0; k < 5; ++k) lamP2[k] = place(np * sizeof(double));
+        tape = place((size_t)sl * TW * (size_t)np * sizeof(double));  // the push's record of a segment
+        for (auto &w : work) w = place(fn * sizeof(double));
+        if (!spin) return;
+        dtab = place(ntab * sizeof(double));
+        tp = place(ntab * sizeof(double));
+        tm = place(ntab * sizeof(double));
+        c1 = place(4 * ctx->g.ld_tab * sizeof(double));
+        Ladev = place(sizeof(double));
+        Lap = place(np * sizeof(double));
+        for (auto &q : segJ) q = place(fn * sizeof(double));
+        for (auto &q : Ystage) q = place(fn * sizeof(double));
+    };
+    layout();
+    // The block stays with the context for the next gradient while it is at most a
+    // sixteenth of the device's memory (mapping 5.5 GB and unmapping it took 27 of
+    // 98 ms); a larger one is given back at once, the kept one by grpic_destroy or
+    // when a call needs more.
+    if (ctx->adj_bytes < need) {
+        cudaFree(ctx->adj_block);
+        ctx->adj_block = nullptr;
+        ctx->adj_bytes = 0;
+        if (cudaMalloc(&ctx->adj_block, need) != cudaSuccess) {
+            cudaGetLastError();
+            ctx->adj_block = nullptr;
+            return GRPIC_ENOMEM;
+        }
+        ctx->adj_bytes = need;
     }
-    for (int k = 0; k < 3; ++k) ok = ok && (lamJ[k] = (double *)dalloc(fn * sizeof(double)));
-    for (int k = 0; k < 5; ++k) {
-        ok = ok && (lamP[k] = (double *)dalloc(np * sizeof(double)));
-        ok = ok && (lamP2[k] = (double *)dalloc(np * sizeof(double)));
-    }
-    // the forward push's record of every step of the current segment
-    const int TW = tape_width(ctx->prm.n_push_iter);
-    double *tape = want ? (double *)dalloc((size_t)ck * TW * (size_t)np * sizeof(double)) : nullptr;
-    ok = ok && (!want || tape);
-    std::vector<double *> work(want ? 24 : 0, nullptr);
-    for (auto &w : work) ok = ok && (w = (double *)dalloc(fn * sizeof(double)));
-    // spin derivative: derivative tables, per-particle parts, the segment's
-    // currents and one update's stage outputs
-    const bool spin = dL_da != nullptr;
-    const int NF = ctx->prm.n_field_iter;
-    const size_t ntab = ctx->slab * T_COUNT;
-    double *dtab = nullptr, *Ladev = nullptr, *Lap = nullptr;
-    std::vector<double *> segJ(spin ? 3 * ck : 0, nullptr), Ystage(spin ? 6 * (NF + 1) : 0, nullptr);
-    if (spin) {
-        ok = ok && (dtab = (double *)dalloc(ntab * sizeof(double)));
-        ok = ok && (Ladev = (double *)dalloc(sizeof(double)));
-        ok = ok && (Lap = (double *)dalloc(np * sizeof(double)));
-        for (auto &q : segJ) ok = ok && (q = (double *)dalloc(fn * sizeof(double)));
-        for (auto &q : Ystage) ok = ok && (q = (double *)dalloc(fn * sizeof(double)));
-    }
-    if (!ok) {
-        cleanup();
-        return GRPIC_ENOMEM;
-    }
+    base = (char *)ctx->adj_block;
+    layout();
+    auto cleanup = [&]() {
+        cudaStreamSynchronize(s);
+        size_t free_b = 0, total = 0;
+        cudaMemGetInfo(&free_b, &total);
+        if (ctx->adj_bytes > total / 16) {
+            cudaFree(ctx->adj_block);
+            ctx->adj_block = nullptr;
+            ctx->adj_bytes = 0;
+        }
+    };
     if (spin) {
         // a-derivatives of the tables by central differences, h = 1e-5 (the
         // quadratures are smooth in a: truncation ~h^2, rounding ~1e-16/h)
         const double h = 1e-5;
-        double *tp = (double *)dalloc(ntab * sizeof(double)), *tm = (double *)dalloc(ntab * sizeof(double));
-        double *c1 = (double *)dalloc(4 * ctx->g.ld_tab * sizeof(double));
-        if (!tp || !tm || !c1 || launch_tables_at(ctx, ctx->g.a + h, tp, c1, s) != cudaSuccess ||
+        if (launch_tables_at(ctx, ctx->g.a + h, tp, c1, s) != cudaSuccess ||
             launch_tables_at(ctx, ctx->g.a - h, tm, c1, s) != cudaSuccess) {
             cleanup();
-            return GRPIC_ENOMEM;
+            return GRPIC_ECUDA;
         }
         central_diff<<<(unsigned)((ntab + 255) / 256), 256, 0, s>>>(tp, tm, 0.5 / h, ntab, dtab);
         cudaMemsetAsync(Ladev, 0, sizeof(double), s);
@@ -1429,7 +1370,6 @@ extern "C" grpic_status grpic_adjoint_grad(grpic_ctx *ctx, const grpic_particles
     void *px[5] = {p0->x1, p0->x2, p0->u1, p0->u2, p0->u3};
     for (int k = 0; k < 5; ++k) cudaMemcpyAsync(W.x[k], px[k], np * sizeof(double), cudaMemcpyDeviceToDevice, s);
     cudaMemcpyAsync(W.tag, p0->tag, np * sizeof(uint32_t), cudaMemcpyDeviceToDevice, s);
-    cudaMemcpyAsync(cnt, &np, sizeof(int64_t), cudaMemcpyHostToDevice, s);
     cudaMemsetAsync(Ldev, 0, sizeof(double), s);
 
     grpic_fields FW;
@@ -1450,22 +1390,6 @@ extern "C" grpic_status grpic_adjoint_grad(grpic_ctx *ctx, const grpic_particles
     PW.u2 = W.x[3];
     PW.u3 = W.x[4];
     PW.tag = W.tag;
-    double *Wf[6];
-    for (int k = 0; k < 6; ++k) Wf[k] = W.F[k];
-    double **dWf = nullptr, **dLamF = nullptr, **dLamF2 = nullptr, **dAux = nullptr, **dSegF = nullptr;
-    ok = upload_ptrs(Wf, 6, &dWf, s) == cudaSuccess && upload_ptrs(lamF, 6, &dLamF, s) == cudaSuccess &&
-         upload_ptrs(lamF2, 6, &dLamF2, s) == cudaSuccess && upload_ptrs(aux, 6, &dAux, s) == cudaSuccess &&
-         cudaMalloc(&dSegF, sizeof(double *) * 6) == cudaSuccess;
-    if (ok) {
-        allocs.push_back(dWf);
-        allocs.push_back(dLamF);
-        allocs.push_back(dLamF2);
-        allocs.push_back(dAux);
-        allocs.push_back(dSegF);
-    } else {
-        cleanup();
-        return GRPIC_ENOMEM;
-    }
     FAdj A{ctx->g.nr, ctx->g.nth, ld, ctx->g.ld_tab, ctx->slab, ctx->tab, ctx->col1d};
     const double wL = 1.0 / nsteps, dth = ctx->g.dth;
     grpic_status st = GRPIC_OK;
@@ -1486,10 +1410,9 @@ extern "C" grpic_status grpic_adjoint_grad(grpic_ctx *ctx, const grpic_particles
     }
     // the last segment, the first the reverse sweep needs, is recorded here
     // (its states, the push's record and, for the spin derivative, its
-    // currents) instead of being recomputed from its checkpoint
-    const int last0 = (nseg - 1) * ck;
+    // currents) instead of being recomputed from a checkpoint
     for (int n = 0; n < nsteps && st == GRPIC_OK; ++n) {
-        if (want && n % ck == 0) copy_state(cks[n / ck], W);
+        if (want && n % ck == 0 && n < last0) copy_state(cks[n / ck], W);
         const bool rec = want && n >= last0;
         const int m = n - last0;
         if (rec && m == 0) copy_state(seg[0], W);
@@ -1500,9 +1423,9 @@ extern "C" grpic_status grpic_adjoint_grad(grpic_ctx *ctx, const grpic_particles
                 for (int k = 0; k < 3; ++k)
                     cudaMemcpyAsync(segJ[3 * m + k], Jw[k], fn * sizeof(double), cudaMemcpyDeviceToDevice, s);
         }
-        flux_kernel<<<1, 256, 0, s>>>(A, dWf, i_horizon, dth, wL, Ldev);
+        flux_kernel<<<1, 256, 0, s>>>(A, six(W.F), i_horizon, dth, wL, Ldev);
         if (spin)  // the objective's own tables at F^{n+1}
-            flux_da<<<(ctx->g.nth + 255) / 256, 256, 0, s>>>(A, dtab, dWf, i_horizon, dth, wL, Ladev);
+            flux_da<<<(ctx->g.nth + 255) / 256, 256, 0, s>>>(A, dtab, six(W.F), i_horizon, dth, wL, Ladev);
     }
     cudaMemcpyAsync(L_out, Ldev, sizeof(double), cudaMemcpyDeviceToHost, s);
     if (!want) {
@@ -1517,33 +1440,10 @@ extern "C" grpic_status grpic_adjoint_grad(grpic_ctx *ctx, const grpic_particles
         return st;
     }
     // ---- reverse sweep -----------------------------------------------------
-    for (int k = 0; k < 6; ++k) cudaMemsetAsync(lamF[k], 0, fn * sizeof(double), s);
+    for (int k = 0; k < 6; ++k) cudaMemsetAsync(lamFa[k], 0, fn * sizeof(double), s);
     for (int k = 0; k < 5; ++k) cudaMemsetAsync(lamP[k], 0, np * sizeof(double), s);
-    double **dptrs[8];
-    double *Jl[3] = {lamJ[0], lamJ[1], lamJ[2]};
-    double *cur_dummy[6] = {0};
-    ok = upload_ptrs(lamF, 6, &dptrs[0], s) == cudaSuccess && upload_ptrs(lamF2, 6, &dptrs[1], s) == cudaSuccess &&
-         upload_ptrs(Jl, 3, &dptrs[2], s) == cudaSuccess && upload_ptrs(&work[0], 6, &dptrs[3], s) == cudaSuccess &&
-         upload_ptrs(&work[6], 6, &dptrs[4], s) == cudaSuccess && upload_ptrs(&work[12], 6, &dptrs[5], s) == cudaSuccess &&
-         upload_ptrs(&work[18], 6, &dptrs[6], s) == cudaSuccess && upload_ptrs(cur_dummy, 6, &dptrs[7], s) == cudaSuccess;
-    if (!ok) {
-        cleanup();
-        return GRPIC_ENOMEM;
-    }
-    for (int k = 0; k < 8; ++k) allocs.push_back(dptrs[k]);
-    SpinField spf{dtab, nullptr, nullptr, nullptr, Ladev};
-    if (spin) {
-        ok = upload_ptrs(Ystage.data(), 6 * (NF + 1), &spf.Y, s) == cudaSuccess;
-        if (ok) allocs.push_back(spf.Y);
-        ok = ok && cudaMalloc(&spf.Xn, sizeof(double *) * 6) == cudaSuccess;
-        if (ok) allocs.push_back(spf.Xn);
-        ok = ok && cudaMalloc(&spf.J, sizeof(double *) * 3) == cudaSuccess;
-        if (ok) allocs.push_back(spf.J);
-        if (!ok) {
-            cleanup();
-            return GRPIC_ENOMEM;
-        }
-    }
+    P6 lamF = six(lamFa), lamF2 = six(lamFb);  // the fields' adjoint and the previous step's
+    SpinField spf{dtab, P6(), P6(), Ystage.data(), Ladev};
     dim3 gfull((ctx->g.ld_tab + 63) / 64, (ctx->g.nth + 1 + 3) / 4), blk(64, 4);
     for (int sgi = nseg - 1; sgi >= 0 && st == GRPIC_OK; --sgi) {
         int n0 = sgi * ck, len = std::min(ck, nsteps - n0);
@@ -1561,10 +1461,9 @@ extern "C" grpic_status grpic_adjoint_grad(grpic_ctx *ctx, const grpic_particles
         }
         for (int m = len - 1; m >= 0 && st == GRPIC_OK; --m) {
             // seed: lamF (adjoint of F^{n+1}) += wL dflux/dF^{n+1}
-            for (int k = 0; k < 6; ++k) cudaMemsetAsync(aux[k], 0, fn * sizeof(double), s);
-            cudaMemcpyAsync(dSegF, seg[m + 1].F, sizeof(double *) * 6, cudaMemcpyHostToDevice, s);
-            flux_seed<<<(ctx->g.nth + 127) / 128, 128, 0, s>>>(A, dSegF, i_horizon, dth, wL, dAux);
-            aux_T<<<gfull, blk, 0, s>>>(A, dAux, dLamF);
+            cudaMemsetAsync(aux[0], 0, 6 * fn * sizeof(double), s);
+            flux_seed<<<(ctx->g.nth + 127) / 128, 128, 0, s>>>(A, six(seg[m + 1].F), i_horizon, dth, wL, six(aux));
+            add_from_h<<<gfull, blk, 0, s>>>(A, six(aux), lamF);
             // fields: lamF -> lamF2 (adjoint of F^n through the field update), lamJ
             if (spin) {
                 // the update of step m again, every stage kept
@@ -1572,10 +1471,10 @@ extern "C" grpic_status grpic_adjoint_grad(grpic_ctx *ctx, const grpic_particles
                     st = GRPIC_ECUDA;
                     break;
                 }
-                cudaMemcpyAsync(spf.Xn, seg[m].F, sizeof(double *) * 6, cudaMemcpyHostToDevice, s);
-                cudaMemcpyAsync(spf.J, &segJ[3 * m], sizeof(double *) * 3, cudaMemcpyHostToDevice, s);
+                spf.Xn = six(seg[m].F);
+                spf.J = six(&segJ[3 * m], 3);
             }
-            st = field_adjoint(ctx, lamF, lamF2, lamJ, work.data(), ld, s, dptrs, spin ? &spf : nullptr);
+            st = field_adjoint(ctx, lamF, lamF2, six(lamJ, 3), work.data(), ld, s, spin ? &spf : nullptr);
             if (st != GRPIC_OK) break;
             // particles
             PAdjArgs P;
@@ -1613,8 +1512,7 @@ extern "C" grpic_status grpic_adjoint_grad(grpic_ctx *ctx, const grpic_particles
             }
             if (cudaGetLastError() != cudaSuccess) st = GRPIC_ECUDA;
             for (int k = 0; k < 5; ++k) std::swap(lamP[k], lamP2[k]);
-            // lamF <- lamF2
-            for (int k = 0; k < 6; ++k) cudaMemcpyAsync(lamF[k], lamF2[k], fn * sizeof(double), cudaMemcpyDeviceToDevice, s);
+            std::swap(lamF, lamF2);
         }
     }
     for (int k = 0; k < 5; ++k) cudaMemcpyAsync(grad_p[k], lamP[k], np * sizeof(double), cudaMemcpyDeviceToDevice, s);

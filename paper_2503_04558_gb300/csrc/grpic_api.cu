@@ -1216,7 +1216,7 @@ void grpic_destroy(grpic_ctx *ctx)
     if (ctx->up_stream) cudaStreamDestroy(ctx->up_stream);
     if (ctx->down_stream) cudaStreamDestroy(ctx->down_stream);
     if (ctx->h_count) cudaFreeHost(ctx->h_count);
-    void *ptrs[] = {ctx->d_spawn, ctx->d_rad, ctx->d_offset_prev, ctx->d_cnt9, ctx->d_sortflag, ctx->rcol, ctx->rcen, ctx->trow, ctx->rcol2, ctx->rowsc, ctx->tab, ctx->col1d, ctx->tab32, ctx->col1d32, ctx->fscratch, ctx->q32, ctx->d_status, ctx->d_keys,
+    void *ptrs[] = {ctx->d_spawn, ctx->d_rad, ctx->d_offset_prev, ctx->d_cnt9, ctx->d_sortflag, ctx->rcol, ctx->rcen, ctx->trow, ctx->rcol2, ctx->rowsc, ctx->tab, ctx->col1d, ctx->tab32, ctx->col1d32, ctx->fscratch, ctx->q32, ctx->adj_block, ctx->d_status, ctx->d_keys,
                     ctx->d_count, ctx->d_offset, ctx->d_cursor, ctx->d_blocksum, ctx->d_perm, ctx->d_bigseg};
     for (void *q : ptrs)
         if (q) cudaFree(q);

@@ -126,6 +126,8 @@ struct grpic_ctx {
     // stencils (launch_quad32, before each push), 6 x (nth+1) x fscratch_ld,
     // allocated with the field scratch
     void *q32;
+    void *adj_block;   // the gradient's scratch, kept between calls (bounded, see grpic_adjoint_grad)
+    size_t adj_bytes;
     char err[256];
 };
 
