@@ -162,10 +162,12 @@ __device__ __forceinline__ void sincos_shift_pair(const df &s0, const df &c0, co
 }
 
 // n correctors in pairs from the predictor: on return the changes of r, theta,
-// u_r, u_theta against x^n; false (nothing kept) where an iterate leaves the range
+// u_r, u_theta against x^n; false (nothing kept) where an iterate leaves the range.
+// note(it, changes) sees each iterate that a right-hand side is taken at.
+template <typename NOTE>
 __device__ __forceinline__ bool correctors_df(const df &a, const df &a2, const df &dt, int n, float eps, double r,
                                               double s0, double c0, const double u[3], const Rhs &f0, double &dr,
-                                              double &dth, double &dur, double &dut)
+                                              double &dth, double &dur, double &dut, const NOTE &note)
 {
     const df R = df_of(r), S0 = df_of(s0), C0 = df_of(c0), U0 = df_of(u[0]), U1 = df_of(u[1]), up = df_of(u[2]);
     const df aup = a * up, h = scale2(dt, 0.5f);
@@ -177,6 +179,7 @@ __device__ __forceinline__ bool correctors_df(const df &a, const df &a2, const d
 #pragma unroll 1
     for (int it = 0; it < n; ++it) {
         if (!(fabsf(dT.hi) < room)) return false;
+        note(it, dR, dT, dV, dW);
         df s, c;
         sincos_shift_pair(S0, C0, dT, s, c);
         RhsDf f;
@@ -405,10 +408,27 @@ __global__ void __launch_bounds__(256) push64_kernel(Push64Args A)
         double rt = fma(dt, f0.xr, r), tt = fma(dt, f0.xt, th);
         double urt = fma(dt, f0.ur, u[0]), utt = fma(dt, f0.ut, u[1]);
         int it = 0;
-        if constexpr (!TAPE) {
+        {
+            // the record's iterates: to FP64's rounding (the changes are a
+            // hundredth of the values), sin and cos from x^n's
+            auto note = [&](int k, const df &dR, const df &dT, const df &dV, const df &dW) {
+                if constexpr (TAPE) {
+                    double *q = tape + (int64_t)(TAPE_IT + 6 * k) * tl;
+                    const double d = double_of(dT);
+                    double st, ct;
+                    sincos_shift<double>(s0, c0, d, st, ct);
+                    q[0] = r + double_of(dR);
+                    q[tl] = th + d;
+                    q[2 * tl] = u[0] + double_of(dV);
+                    q[3 * tl] = u[1] + double_of(dW);
+                    q[4 * tl] = st;
+                    q[5 * tl] = ct;
+                }
+            };
             double dr, dth, dur, dut;
             if (A.pairs && A.hf * float_of_pos(fabs(f0.xp)) < PAIR_MAX_ANGLE &&
-                correctors_df(A.a_df, A.a2_df, A.dt_df, A.n_iter - 1, (float)eps, r, s0, c0, u, f0, dr, dth, dur, dut)) {
+                correctors_df(A.a_df, A.a2_df, A.dt_df, A.n_iter - 1, (float)eps, r, s0, c0, u, f0, dr, dth, dur, dut,
+                              note)) {
                 rt = r + dr;
                 tt = th + dth;
                 urt = u[0] + dur;
