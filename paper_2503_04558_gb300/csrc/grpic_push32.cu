@@ -629,14 +629,18 @@ __device__ __forceinline__ void push_slot(const Push32Args &A, const IX p, const
     float o1 = 0, o2 = 0, x2in = 0, u[3] = {0, 0, 0};
     if (p < nx) {
         const IX src = permuted ? (IX)A.perm[p] : p;
+        // all of them at once, also a dead slot's: the tag first would put
+        // another memory latency in front of the rest (2048^2 step 43.8 ->
+        // 42.6 ms, 512^2 2.07 -> 2.00 ms).  A dead slot's values are nobody's:
+        // they travel with it until the next placement drops it.
         tag = A.in_tag[src];
+        cellk = A.in_cell[src];
+        o1 = A.in_o1[src];
+        o2 = x2in = A.in_o2[src];
+        u[0] = A.in_u1[src];
+        u[1] = A.in_u2[src];
+        u[2] = A.in_u3[src];
         if (!(tag & DEAD)) {
-            cellk = A.in_cell[src];
-            o1 = A.in_o1[src];
-            o2 = x2in = A.in_o2[src];
-            u[0] = A.in_u1[src];
-            u[1] = A.in_u2[src];
-            u[2] = A.in_u3[src];
             bool ok = cellk >= 0 && cellk < ncell && o1 >= 0.0f && o1 <= 1.0f && o2 >= 0.0f && o2 <= 1.0f &&
                       isfinite(u[0]) && isfinite(u[1]) && isfinite(u[2]);
             if (ok) {
