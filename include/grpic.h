@@ -374,8 +374,8 @@ grpic_status grpic_adjoint_field_step(grpic_ctx *ctx, const grpic_fields *lam_in
  *   dL_da: NULL or a host double: the derivative of L with respect to the
  *        spin a at fixed step-0 state (p0, f0), fixed grid (r_in, r_out,
  *        n_r, n_theta), dt and i_horizon.  It collects the metric of every
- *        push (Boris and geodesic right-hand sides, exactly: a third dual
- *        slot in their hand-written reverse passes), the tables of every
+ *        push (Boris and geodesic right-hand sides, exactly: through a^2
+ *        and a in their hand-written reverse passes), the tables of every
  *        field update and of the objective (face-area inverses and metric
  *        products of App. B) contracted with the stage adjoints, the tables'
  *        a-derivatives taken by a central difference h = 1e-5 of the

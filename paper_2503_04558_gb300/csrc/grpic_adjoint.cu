@@ -8,17 +8,24 @@
 //   * seed   lambda_F^{n+1} += dL/dF^{n+1}  (through the auxiliary fields);
 //   * fields the field update is linear in (F^n, J): its transpose runs the
 //            predictor-corrector stages backwards with the transposed circulation
-//            and auxiliary-field stencils (scatter with atomics), the boundary
-//            copies transposed into their source cells;
+//            and auxiliary-field stencils, each point gathering what its readers
+//            hand back (two launches a stage, no atomics), the boundary copies
+//            transposed into their source cells;
 //   * particles for every particle: the transpose of the deposit (derivatives of
 //            the piecewise-linear CIC weights), the axis reflection, the geodesic
 //            step (the predictor and correctors as run, transposed one by one,
 //            or the implicit-function theorem at the converged trapezoid,
 //            (I - dt/2 dF/dy)^T w = lambda, a 5x5 solve), the Boris step and the
 //            interpolation (scatter of lambda_E into lambda_F).  Vector-Jacobian
-//            products of the right-hand side are a hand-written reverse pass;
-//            the metric's derivatives and the other local Jacobians come from
-//            forward-mode dual numbers through the same metric code.
+//            products of the right-hand side and of the Boris step are reverse
+//            passes written out through the push's point quantities; the window's
+//            transpose interpolates the adjoint currents.  Forward-mode dual
+//            numbers through the metric code give the full Jacobian that the
+//            implicit-function form needs.
+//            Bound by the FP64 pipe (88 % busy; 1120 of its instructions a
+//            particle; 4.24 ms for 2e6 particles, 9.5 ms with dual numbers and
+//            row-by-row window contractions; the early correctors' transposes in
+//            double-FP32 pairs: slower, 8 warps per SM do not hide their chains).
 // Recompute checkpoints every `checkpoint_every` steps bound the memory; the
 // segment's recompute runs the FP64 push in its recording form, so the
 // particle adjoint reads the Boris output and the corrector iterates (with

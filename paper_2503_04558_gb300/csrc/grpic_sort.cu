@@ -29,11 +29,12 @@
 // and step 5's gather moves the data, as for the general path.  Placing only
 // the indices keeps the per-cell bookkeeping off the particle data: the
 // gather's reads are nearly sequential runs and its writes sequential.
-// The count pass checks the precondition (every key a neighbour of its
-// segment, live count = the previous sort's) and raises a device flag when
-// it fails; the general kernels then run instead.  Every kernel of both paths
-// reads the flag and strides over its work with a fixed grid, so the path
-// not taken costs one flag read per block.
+// Where the push counted (6) itself, reading through the last sort's permutation,
+// the precondition holds by construction and only 7 and 8 are launched.  Elsewhere
+// a count pass checks it (every key a neighbour of its segment, live count = the
+// previous sort's) and raises a device flag when it fails; the general kernels then
+// run instead.  Every kernel of both paths reads the flag and strides over its work
+// with a fixed grid, so the path not taken costs one flag read per block.
 #include "grpic_internal.cuh"
 
 #include <algorithm>
