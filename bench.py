@@ -53,35 +53,37 @@ B0 = 1.0
 # kernels (flop = 2 FMA + MUL + ADD of the SASS instruction counters) in one
 # capture of a smaller case of the same workload (same spin, radial range and
 # island fraction), and scaled to a launch by the number of particles.
-PUSH64_FP64_FLOP = 1039.3   # FP64 push, 512^2 x 64 ppc split monopole
-PUSH64_DRAM_B = 95.6        # the same capture: DRAM bytes per particle (read + write)
-PUSH32_FP32_FLOP = 594.2    # FP32-form push, 1024^2 x 64 ppc split monopole
+PUSH64_FP64_FLOP = 554.2    # FP64 push, 512^2 x 64 ppc split monopole (its early correctors run in FP32 pairs)
+PUSH64_DRAM_B = 95.3        # the same capture: DRAM bytes per particle (read + write)
+PUSH32_FP32_FLOP = 557.1    # FP32-form push, 1024^2 x 64 ppc split monopole
 # the same capture: instructions issued per particle (warp instructions x 32)
 # and DRAM bytes per particle (read + write)
-PUSH32_INST = 1029.8
-PUSH32_DRAM_B = 68.0
+PUSH32_INST = 1020.1
+PUSH32_DRAM_B = 66.8
 # batched 1D lines, b1_kernel with the cascade running (256 lines x 4096 cells):
 # instructions issued per particle-step (warp instructions x 32) and DRAM
 # bytes per particle-step; algorithmic bytes: the particle record (cell, offset,
 # u_r, u_phi, tag as 4 B each, id 8 B) read and written once per step
-B1_INST = 1037.0
-B1_DRAM_B = 51.7
+B1_INST = 960.6
+B1_DRAM_B = 51.8
 # the same kernel in the grown-cascade state (64 lines x 4096 cells, 10^U(4,5.5)
 # particles per line of charge weight 1/20, after 600 steps: appends running)
-B1G_INST = 1052.8
-B1G_DRAM_B = 53.1
+B1G_INST = 978.1
+B1G_DRAM_B = 53.4
 B1_ALG_B = 2 * 28
 # the widened rows' push kernels, counted the same way: the FP32 push with
 # Vay's update (1024^2 x 64 ppc), the FP64 push with the cubic shape (512^2 x
 # 64 ppc), the FP64 push with photon emission and conversion decisions (512^2
 # x 16 ppc, Wald a = 0.99, B0 = 500)
-VAY32_FP32_FLOP = 651.8
-VAY32_INST = 1107.7
-CUBIC64_FP64_FLOP = 1471.4
-RAD64_FP64_FLOP = 1248.5
+VAY32_FP32_FLOP = 614.8
+VAY32_INST = 1095.7
+CUBIC64_FP64_FLOP = 984.3
+RAD64_FP64_FLOP = 644.3
 VAY_COUNT = "ncu SASS counters, FP32-form push with Vay's update, 1024^2 x 64 ppc"
 CUBIC_COUNT = "ncu SASS counters, FP64 push with the cubic shape, 512^2 x 64 ppc"
 RAD_COUNT = "ncu SASS counters, FP64 push with emission/conversion decisions, 512^2 x 16 ppc"
+# cells from which the sort's scan of the destinations takes a third launch
+SORT_TILES = 1024 * 1024
 
 
 _ALU = None
@@ -1156,13 +1158,16 @@ def main():
                 "particle_statuses": h["particle_statuses"],
                 "roofline": h["roofline"], "clocks": h["clocks"], "measured_alu_peaks": measured_alu(),
                 # per step: push (FP32: with the fields' stencil quads built
-                # first), the field update (FP32: fused launches of four
-                # stages; FP64: 1 + n_field_iter stage launches), 12 sort kernels
-                # (count, destinations, histogram pair, 3 scan, bases, placement and
-                # the general path's 3, which return at once) -- the count only
-                # in the first step, later pushes count -- and one gather per call
+                # first), the field update (FP32: launches of four stages on
+                # tiles; FP64: 1 + n_field_iter stage launches) and the sort: 11
+                # kernels in the first step (count, destinations, histogram pair,
+                # 3 scan, placement and the general path's 3, which return at
+                # once); later pushes count, which leaves the destinations with
+                # their scan (3; 2 on grids below SORT_TILES cells) and the
+                # placement.  One gather per call
                 "gpu_launches": args.steps * (1 + ((1 + (1 + cfg.n_field_iter + 3) // 4) if head_prec == 32 else
-                                                   1 + cfg.n_field_iter) + 12) - (args.steps - 1) + 1,
+                                                   1 + cfg.n_field_iter)) + 11 + (args.steps - 1) *
+                                (4 if h["cells"] + 1 > SORT_TILES else 3) + 1,
                 "e2e": res["e2e"]}
         if second is not None:
             s2 = grpic_summary(second, args, world, 64)
