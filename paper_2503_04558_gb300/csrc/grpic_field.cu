@@ -26,27 +26,45 @@ namespace {
 // to the neighbours through shared memory: first the products whose column
 // neighbours the auxiliary fields average (products()), then the auxiliary
 // fields E_i, H_i themselves (auxiliary()), then the circulations (circulation()),
-// so no table value of a neighbour is read.  The predictor leaves the part of
-// the correctors that does not change, the base
+// so no table value of a neighbour is read.
+//
+// FP64: the predictor leaves the part of the correctors that does not change,
+// the base
 //   X^n + dt (alpha_s C(X^n) - J / A),
 // and a corrector is base + (dt beta_s / A) circ(X): X^n, C^n and J are not read
 // again.  52 operations per point and stage (122 when each point evaluated its
 // neighbours' auxiliary fields and combined X^n, C^n and J in every stage).
-// One update (8 stages): FP32 2048^2 1.29 -> 0.63 ms, FP64 1024^2 2.44 -> 1.15
-// ms (82 % of the FP64 pipe's cycles); FP64 128^2 0.128 -> 0.066 ms, FP32 128^2
-// 0.071 -> 0.016 ms.
-// The fused multiply-adds are written out, so both kernels round alike.
+//
+// FP32: the order of the roundings is fixed, operation by operation:
+//   products t x of a pair: fma(own t, own x, round(neighbour's t x)), halved;
+//   auxiliary fields: fma(t, x, half pair), then -+ the second half pair;
+//   C = round(circ / A), Jd = round(J / A);
+//   predictor: fma(dt, C - Jd, X^n);
+//   corrector: fma(-Jd, dt, fma(dt, m, X^n)), m = alpha_s C^n + beta_s C with one of
+//   the products inside the fused multiply-add (FieldArgs::lead).
+// A step's currents amplify the last bit of the fields: next to the axis J^phi is
+// decided by a few particles, and a field off by one rounding moves them by up to
+// 1e-3 of their size.  With the order fixed a run's fields are the same bits on
+// every launch shape, and the same as before the shapes were changed.  (Folding
+// alpha_s, J and dt / A into a base as in FP64: 0.63 ms an update at 2048^2, but two
+// steps at that size then ended with J^phi 2.4e-4 off.)
+// One update (8 stages): FP32 2048^2 1.29 -> 0.81 ms, FP64 1024^2 2.44 -> 1.15
+// ms (82 % of the FP64 pipe's cycles); FP64 128^2 0.128 -> 0.066 ms.
 template <typename T>
 struct FieldArgs {
     int nr, nth, ldt, ld;
     size_t slab;
-    T dt, as, dtbs, dth;
+    T dt, as, bs, dtbs, dth;
     const T *tab;
     const T *col1d;  // dr_prim, dr_dual, damp_int, damp_half
     const T *Xi[6];  // the iterate at the launch's first stage
     T *Xo[6];        // the iterate after its last one
-    T *Bs[6];        // the base (written by the first launch, read by the others)
+    T *Bs[6];        // FP64: the base; FP32: C^n, times alpha_s if `lead` (written by the
+                     // first launch, read by the others)
+    const T *Xn[6];  // FP32: X^n for the launches after the first
+    T *Xs[6];        // FP32 tiles: a copy of X^n, written by the first launch
     const T *J[3];
+    int lead;        // FP32: fma(beta_s, C, alpha_s C^n), else fma(alpha_s, C^n, beta_s C)
     int j_lo, j_hi;  // the rows updated
     int rows;        // strip kernel: rows per CTA
     int ns;          // tile kernel: stages of this launch
@@ -99,6 +117,37 @@ __device__ __forceinline__ void auxiliary(const T *K, const T *X, const T *S, in
     E[5 * m + o] = fmat(h, fmat(K[6], X[0], fmat(K[7], X[4], S[5 * n + el])), K[13] * X[2]);
 }
 
+// FP32: the same with every pair's products apart, K[0..7] halved
+__device__ __forceinline__ void products(const float *K, const float *X, float *S, int n, int e)
+{
+    S[e] = K[0] * X[5];
+    S[n + e] = K[1] * X[2];
+    S[2 * n + e] = K[2] * X[3];
+    S[3 * n + e] = K[3] * X[1];
+    S[4 * n + e] = K[4] * X[2];
+    S[5 * n + e] = K[5] * X[5];
+    S[6 * n + e] = K[6] * X[0];
+    S[7 * n + e] = K[7] * X[4];
+}
+__device__ __forceinline__ void auxiliary(const float *K, const float *X, const float *S, int n, int el, int er, float *E,
+                                          int m, int o)
+{
+    E[o] = fmaf(K[8], X[3], fmaf(K[0], X[5], S[el]));
+    E[m + o] = fmaf(K[9], X[4], fmaf(K[1], X[2], S[n + er]));
+    E[2 * m + o] = __fsub_rn(fmaf(K[10], X[5], fmaf(K[2], X[3], S[2 * n + er])), fmaf(K[3], X[1], S[3 * n + er]));
+    E[3 * m + o] = fmaf(K[11], X[0], fmaf(K[4], X[2], S[4 * n + er]));
+    E[4 * m + o] = fmaf(K[12], X[1], -fmaf(K[5], X[5], S[5 * n + el]));
+    E[5 * m + o] = __fadd_rn(fmaf(K[13], X[2], fmaf(K[6], X[0], S[6 * n + el])), fmaf(K[7], X[4], S[7 * n + el]));
+}
+template <typename T>
+constexpr int N_PROD = sizeof(T) == 4 ? 8 : 6;
+// a coefficient as the products take it
+template <typename T>
+__device__ __forceinline__ T coef_value(int k, T v)
+{
+    return sizeof(T) == 4 && k < 8 ? T(0.5) * v : v;
+}
+
 // the circulations of Eqs. D-update, B-update (not yet divided by the areas)
 // from the auxiliary fields at the point o, its column neighbours l, r and its
 // row neighbours d (below), u (above).  Beyond the axis rows H_phi is zero (its
@@ -116,7 +165,24 @@ __device__ __forceinline__ void circulation(const T *E, int m, int o, int l, int
     C[5] = fmat(E[4 * m + o] - E[4 * m + r], dth, (E[3 * m + u] - E[3 * m + o]) * drp);
 }
 
-// the predictor at one component: X^n -> X~ and the base B
+// FP32: the predictor at one component (J: its current, 0 for B), X^n -> X~; Q: C^n
+// as the correctors take it, Jd: J / A
+__device__ __forceinline__ void predict(float C, float W, float J, const FieldArgs<float> &A, float &X, float &Q, float &Jd)
+{
+    const float Cn = __fmul_rn(C, W);
+    Jd = __fmul_rn(J, W);
+    Q = A.lead ? __fmul_rn(A.as, Cn) : Cn;
+    X = fmaf(A.dt, __fsub_rn(Cn, Jd), X);
+}
+// ... and a corrector
+__device__ __forceinline__ float correct(float C, float W, float Q, float Xn, float Jd, const FieldArgs<float> &A)
+{
+    const float c = __fmul_rn(C, W);
+    const float m = A.lead ? fmaf(A.bs, c, Q) : fmaf(A.as, Q, __fmul_rn(A.bs, c));
+    return fmaf(-Jd, A.dt, fmaf(A.dt, m, Xn));
+}
+
+// FP64: the predictor at one component: X^n -> X~ and the base B
 template <typename T>
 __device__ __forceinline__ void predict(T C, T W, T J, T dt, T as, T &X, T &B)
 {
@@ -137,32 +203,35 @@ __device__ __forceinline__ void put_value(T *row, int c, int i, int last, int ld
 }
 
 // NS consecutive stages per launch on a BW x BH tile of points, P of them per
-// thread (a fixed column, rows RS apart): the points' iterate, base and
-// coefficients stay in registers over the launch.  A stage reads one point
-// beyond the one it writes, so the outer NS points of the tile are a halo that
-// neighbouring CTAs compute too; the last launch writes the caller's arrays
-// (no CTA reads X^n any more).  Points that a component does not update (guard
-// columns, rows beyond the axis) carry W = 0 and hold their value.  For FP32,
-// where issue (47 % of the slots) and the loads at a tile's start bound it (the
-// next tile's lines are asked for ahead: 0.66 -> 0.63 ms per update at 2048^2;
-// 768 threads of two points each: the same); FP64 is bound by its pipe, which
-// the halo's second computation would load.
-template <typename T, int BW, int BH, int P, int NS, int MINB, bool FIRST>
-__global__ void __launch_bounds__(BW *BH / P, MINB) field_tile_kernel(const __grid_constant__ FieldArgs<T> A)
+// thread (a fixed column, rows RS apart): the points' iterate, inverse areas and
+// coefficients stay in registers over the launch, X^n, C^n and J / A in shared
+// memory (each thread reads its own).  A stage reads one point beyond the one it
+// writes, so the outer NS points of the tile are a halo that neighbouring CTAs
+// compute too.  The first launch leaves a copy of X^n for the later ones, so that
+// the last one can write the caller's arrays.  Points that a component does not
+// update (rows beyond the axis) carry W = 0 and X^n = 0; guard columns are set from
+// the physical ones after each stage.  FP32 only: issue and the loads at a tile's
+// start bound it (the next tile's lines are asked for ahead); FP64 is bound by its
+// pipe, which the halo's second computation would load.
+template <int BW, int BH, int P, int NS, int MINB, bool FIRST>
+__global__ void __launch_bounds__(BW *BH / P, MINB) field_tile_kernel(const __grid_constant__ FieldArgs<float> A)
 {
     constexpr int NT = BW * BH / P, RS = NT / BW, OW = BW - 2 * NS, OH = BH - 2 * NS, BOX = BW * BH;
     static_assert(NT % BW == 0 && NT % 32 == 0, "a thread's points share their column");
     extern __shared__ __align__(16) unsigned char field_smem[];
-    T *const S = reinterpret_cast<T *>(field_smem);
-    T *const E = S + 6 * BOX;
-    T *const Gd = E + 6 * BOX;  // guard copies, 12 x BH
+    float *const S = reinterpret_cast<float *>(field_smem);
+    float *const E = S + N_PROD<float> * BOX;
+    float *const Q = E + 6 * BOX;    // C^n as the correctors take it
+    float *const XN = Q + 6 * BOX;   // X^n
+    float *const JD = XN + 6 * BOX;  // J / A
+    float *const Gd = JD + 3 * BOX;  // guard copies, 12 x BH
     const int nr = A.nr, nth = A.nth;
     const int bc = threadIdx.x % BW, br0 = threadIdx.x / BW;
     const int c0 = (int)blockIdx.x * OW - NS, r0 = A.j_lo + (int)blockIdx.y * OH - NS;
     const int c = c0 + bc, i = c - NG;
     const bool col_in = c >= 0 && c < A.ldt;
     const bool ph_i = i >= 0 && i <= nr, ph_h = i >= 0 && i <= nr - 1;  // integer, half-r components
-    T drp = T(0), drd = T(0), dmi = T(1), dmh = T(1);
+    float drp = 0.0f, drd = 0.0f, dmi = 1.0f, dmh = 1.0f;
     if (col_in) {
         drp = __ldg(A.col1d + c);
         drd = __ldg(A.col1d + A.ldt + c);
@@ -170,43 +239,44 @@ __global__ void __launch_bounds__(BW *BH / P, MINB) field_tile_kernel(const __gr
         dmh = __ldg(A.col1d + 3 * A.ldt + c);
     }
     // the lines of the tile that this SM is likely to take next, into L2
-    for (int t = threadIdx.x; t < (FIRST ? 26 : 32) * BH; t += NT) {
+    for (int t = threadIdx.x; t < (FIRST ? 26 : 41) * BH; t += NT) {
         const int next = (int)(blockIdx.y * gridDim.x + blockIdx.x) + A.ahead, q = t / BH;
         const int j = next / (int)gridDim.x * OH - NS + t % BH, col = max(next % (int)gridDim.x * OW - NS, 0);
         if (j < 0 || j > nth) continue;
-        const T *row = q < 20 ? A.tab + (q < 6 ? q : q + 6) * A.slab + (unsigned)(j * A.ldt)
-                              : (q < 26 ? A.Xi[q - 20] : A.Bs[q - 26]) + (unsigned)(j * A.ld);
+        const float *row = q < 20   ? A.tab + (q < 6 ? q : q + 6) * A.slab + (unsigned)(j * A.ldt)
+                           : q < 26 ? A.Xi[q - 20] + (unsigned)(j * A.ld)
+                           : q < 32 ? A.Bs[q - 26] + (unsigned)(j * A.ld)
+                           : q < 38 ? A.Xn[q - 32] + (unsigned)(j * A.ld)
+                                    : A.J[q - 38] + (unsigned)(j * A.ld);
         asm volatile("prefetch.global.L2 [%0];" ::"l"(row + min(col, A.ldt - 1)));
         asm volatile("prefetch.global.L2 [%0];" ::"l"(row + min(col + 32, A.ldt - 1)));
     }
-    T X[P][6], B[P][6], W[P][6], K[P][14];
+    float X[P][6], W[P][6], K[P][14];
 #pragma unroll
     for (int p = 0; p < P; ++p) {
-        const int j = r0 + br0 + p * RS;
+        const int j = r0 + br0 + p * RS, e = threadIdx.x + p * NT;
         const bool in = col_in && j >= 0 && j <= nth, axis = j == 0 || j == nth;
         const unsigned q = (unsigned)(j * A.ld + c), qt = (unsigned)(j * A.ldt + c);
 #pragma unroll
         for (int k = 0; k < 6; ++k) {
             const bool row = in && !(half_t(k) && j == nth);
             const bool upd = row && (half_r(k) ? ph_h : ph_i) && !((k == 2 || k == 4) && axis);
-            X[p][k] = row ? __ldg(A.Xi[k] + q) : T(0);
-            W[p][k] = upd ? __ldg(A.tab + inv_area(k) * A.slab + qt) : T(0);
+            X[p][k] = row ? __ldg(A.Xi[k] + q) : 0.0f;
+            W[p][k] = upd ? __ldg(A.tab + inv_area(k) * A.slab + qt) : 0.0f;
+            XN[k * BOX + e] = !upd ? 0.0f : (FIRST ? X[p][k] : __ldg(A.Xn[k] + q));
             if (!FIRST) {
-                B[p][k] = upd ? __ldg(A.Bs[k] + q) : X[p][k];
-                W[p][k] *= A.dtbs;
+                Q[k * BOX + e] = upd ? __ldg(A.Bs[k] + q) : 0.0f;
+                if (k < 3) JD[k * BOX + e] = upd ? __fmul_rn(__ldg(A.J[k < 3 ? k : 0] + q), W[p][k]) : 0.0f;
             }
         }
 #pragma unroll
-        for (int k = 0; k < 14; ++k) K[p][k] = in ? __ldg(A.tab + coef(k) * A.slab + qt) : T(0);
+        for (int k = 0; k < 14; ++k) K[p][k] = in ? coef_value(k, __ldg(A.tab + coef(k) * A.slab + qt)) : 0.0f;
     }
     const int dl = bc > 0 ? 1 : 0, dr = bc < BW - 1 ? 1 : 0;
     const int dd = br0 > 0 ? BW : 0, du = br0 < RS - 1 ? BW : 0;  // of a thread's first and last point
-    auto circ_of = [&](T(&C)[P][6]) {
+    auto fields = [&]() {
 #pragma unroll
-        for (int p = 0; p < P; ++p) {
-            const int e = threadIdx.x + p * NT;
-            products(K[p], X[p], S, BOX, e);
-        }
+        for (int p = 0; p < P; ++p) products(K[p], X[p], S, BOX, (int)threadIdx.x + p * NT);
         __syncthreads();
 #pragma unroll
         for (int p = 0; p < P; ++p) {
@@ -214,12 +284,10 @@ __global__ void __launch_bounds__(BW *BH / P, MINB) field_tile_kernel(const __gr
             auxiliary(K[p], X[p], S, BOX, e - dl, e + dr, E, BOX, e);
         }
         __syncthreads();
-#pragma unroll
-        for (int p = 0; p < P; ++p) {
-            const int e = threadIdx.x + p * NT;
-            circulation(E, BOX, e, e - dl, e + dr, e - (p == 0 ? dd : BW), e + (p == P - 1 ? du : BW), A.dth, drp, drd,
-                        C[p]);
-        }
+    };
+    auto circ_of = [&](int p, float(&C)[6]) {
+        const int e = threadIdx.x + p * NT;
+        circulation(E, BOX, e, e - dl, e + dr, e - (p == 0 ? dd : BW), e + (p == P - 1 ? du : BW), A.dth, drp, drd, C);
     };
     // guard columns i = -1, n_r (half-r components) and n_r + 1: zero-derivative
     // copies of the first / last physical column
@@ -241,35 +309,42 @@ __global__ void __launch_bounds__(BW *BH / P, MINB) field_tile_kernel(const __gr
             const int br = br0 + p * RS;
 #pragma unroll
             for (int k = 0; k < 6; ++k) {
-                if (i == -1) B[p][k] = X[p][k] = Gd[k * BH + br];
-                if (i == nr + 1 || (i == nr && half_r(k))) B[p][k] = X[p][k] = Gd[(6 + k) * BH + br];
+                if (i == -1) X[p][k] = Gd[k * BH + br];
+                if (i == nr + 1 || (i == nr && half_r(k))) X[p][k] = Gd[(6 + k) * BH + br];
             }
         }
     };
     int st = 0;
-    T C[P][6];
     if constexpr (FIRST) {
-        circ_of(C);
+        fields();
 #pragma unroll
         for (int p = 0; p < P; ++p) {
-            const int j = r0 + br0 + p * RS;
-            const bool axis = j == 0 || j == nth;
+            const int j = r0 + br0 + p * RS, e = threadIdx.x + p * NT;
+            float C[6];
+            circ_of(p, C);
 #pragma unroll
             for (int k = 0; k < 6; ++k) {
-                const T J = k < 3 && W[p][k] != T(0) ? __ldg(A.J[k < 3 ? k : 0] + (unsigned)(j * A.ld + c)) : T(0);
-                predict(C[p][k], W[p][k], J, A.dt, A.as, X[p][k], B[p][k]);
-                W[p][k] *= A.dtbs;
-                if ((k == 2 || k == 4) && axis) X[p][k] = B[p][k] = T(0);  // D^ph, B^th on the axis
+                float J = 0.0f, q, jd;
+                if (k < 3 && W[p][k] != 0.0f) J = __ldg(A.J[k < 3 ? k : 0] + (unsigned)(j * A.ld + c));
+                predict(C[k], W[p][k], J, A, X[p][k], q, jd);
+                if ((k == 2 || k == 4) && (j == 0 || j == nth)) X[p][k] = 0.0f;  // D^ph, B^th on the axis
+                Q[k * BOX + e] = q;
+                if (k < 3) JD[k * BOX + e] = jd;
             }
         }
         if (++st < A.ns) guards();
     }
     while (st < A.ns) {
-        circ_of(C);
+        fields();
 #pragma unroll
-        for (int p = 0; p < P; ++p)
+        for (int p = 0; p < P; ++p) {
+            const int e = threadIdx.x + p * NT;
+            float C[6];
+            circ_of(p, C);
 #pragma unroll
-            for (int k = 0; k < 6; ++k) X[p][k] = fmat(C[p][k], W[p][k], B[p][k]);
+            for (int k = 0; k < 6; ++k)
+                X[p][k] = correct(C[k], W[p][k], Q[k * BOX + e], XN[k * BOX + e], k < 3 ? JD[(k < 3 ? k : 0) * BOX + e] : 0.0f, A);
+        }
         if (++st < A.ns) guards();
     }
     if (A.last)
@@ -281,14 +356,17 @@ __global__ void __launch_bounds__(BW *BH / P, MINB) field_tile_kernel(const __gr
     if (bc < NS || bc >= NS + OW || !ph_i) return;
 #pragma unroll
     for (int p = 0; p < P; ++p) {
-        const int br = br0 + p * RS, j = r0 + br;
+        const int br = br0 + p * RS, j = r0 + br, e = threadIdx.x + p * NT;
         if (br < NS || br >= NS + OH || j > nth) continue;
         const size_t row = (size_t)j * A.ld;
 #pragma unroll
         for (int k = 0; k < 6; ++k) {
             if ((half_r(k) && !ph_h) || (half_t(k) && j == nth)) continue;
             put_value(A.Xo[k] + row, c, i, half_r(k) ? nr - 1 : nr, A.ldt, X[p][k]);
-            if (FIRST && !A.last) A.Bs[k][row + c] = B[p][k];
+            if (FIRST && A.Xs[k]) {
+                A.Bs[k][row + c] = Q[k * BOX + e];
+                A.Xs[k][row + c] = XN[k * BOX + e];
+            }
         }
     }
 }
@@ -304,7 +382,7 @@ __global__ void __launch_bounds__(BW *RT, RES) field_strip_kernel(const __grid_c
 {
     constexpr int RING = RT <= 2 ? 4 : (RT <= 6 ? 8 : 16), NE = BW * RING, NP = BW * RT;
     static_assert(RING >= RT + 2, "the update reads two rows above the new ones");
-    __shared__ T S[6 * NP], E[6 * NE];
+    __shared__ T S[N_PROD<T> * NP], E[6 * NE];
     const int nr = A.nr, nth = A.nth;
     const int bc = threadIdx.x % BW, rt = threadIdx.x / BW;
     const int c = (int)blockIdx.x * (BW - 2) - 1 + bc, i = c - NG;
@@ -329,7 +407,7 @@ __global__ void __launch_bounds__(BW *RT, RES) field_strip_kernel(const __grid_c
 #pragma unroll
         for (int k = 0; k < 6; ++k) X[k] = in && !(half_t(k) && j == nth) ? __ldg(A.Xi[k] + q) : T(0);
 #pragma unroll
-        for (int k = 0; k < 14; ++k) K[k] = in ? __ldg(A.tab + coef(k) * A.slab + qt) : T(0);
+        for (int k = 0; k < 14; ++k) K[k] = in ? coef_value(k, __ldg(A.tab + coef(k) * A.slab + qt)) : T(0);
     };
     load(ja - 1 + rt);
     for (int jt = ja - 1; jt <= jb; jt += RT) {
@@ -339,12 +417,13 @@ __global__ void __launch_bounds__(BW *RT, RES) field_strip_kernel(const __grid_c
         const int ju = j - 1;
         const bool upd = mine && ju >= ja && ju < jb, axis = ju == 0 || ju == nth;
         const unsigned q = (unsigned)(ju * A.ld + c);
-        T W[6], B[6];
+        T W[6], B[6], XN[6];
 #pragma unroll
         for (int k = 0; k < 6; ++k) {
             const bool on = upd && !(half_r(k) && !ph_h) && !(half_t(k) && ju == nth) && !((k == 2 || k == 4) && axis);
             W[k] = on ? __ldg(A.tab + inv_area(k) * A.slab + (unsigned)(ju * A.ldt + c)) : T(0);
-            B[k] = on ? __ldg((FIRST ? A.Xi[k] : A.Bs[k]) + q) : T(0);  // X^n or the base
+            B[k] = on ? __ldg((FIRST ? A.Xi[k] : A.Bs[k]) + q) : T(0);  // X^n or what the predictor left
+            if (sizeof(T) == 4 && !FIRST) XN[k] = on ? __ldg(A.Xn[k] + q) : T(0);
         }
         products(K, X, S, NP, (int)threadIdx.x);
         __syncthreads();
@@ -361,10 +440,19 @@ __global__ void __launch_bounds__(BW *RT, RES) field_strip_kernel(const __grid_c
             for (int k = 0; k < 6; ++k) {
                 if ((half_r(k) && !ph_h) || (half_t(k) && ju == nth)) continue;
                 T v, b = T(0);
+                T J = T(0);
+                if ((FIRST || sizeof(T) == 4) && k < 3) J = __ldg(A.J[k < 3 ? k : 0] + q);
                 if constexpr (FIRST) {
                     v = B[k];
-                    predict(C[k], W[k], k < 3 ? __ldg(A.J[k < 3 ? k : 0] + q) : T(0), A.dt, A.as, v, b);
+                    if constexpr (sizeof(T) == 4) {
+                        float jd;
+                        predict(C[k], W[k], J, A, v, b, jd);
+                    } else {
+                        predict(C[k], W[k], J, A.dt, A.as, v, b);
+                    }
                     if ((k == 2 || k == 4) && axis) v = b = T(0);
+                } else if constexpr (sizeof(T) == 4) {
+                    v = (k == 2 || k == 4) && axis ? 0.0f : correct(C[k], W[k], B[k], XN[k], __fmul_rn(J, W[k]), A);
                 } else {
                     v = fmat(C[k], W[k] * A.dtbs, B[k]);
                 }
@@ -384,25 +472,25 @@ T *fslot(grpic_ctx *ctx, int k, int64_t ld)
 }
 
 // a launch shape of the tile kernel
-template <typename T, int BW, int BH, int P, int NS, int MINB>
+template <int BW, int BH, int P, int NS, int MINB>
 struct Tiles {
     static constexpr int OW = BW - 2 * NS, OH = BH - 2 * NS, threads = BW * BH / P, stages = NS;
-    static constexpr int smem = 12 * (BW * BH + BH) * (int)sizeof(T);
-    static dim3 grid(const FieldArgs<T> &A) { return dim3((A.ldt + OW - 1) / OW, (A.j_hi - A.j_lo + OH - 1) / OH); }
-    static cudaError_t setup(FieldArgs<T> &A, int sms)
+    static constexpr int smem = ((N_PROD<float> + 6 + 15) * BW * BH + 12 * BH) * (int)sizeof(float);
+    static dim3 grid(const FieldArgs<float> &A) { return dim3((A.ldt + OW - 1) / OW, (A.j_hi - A.j_lo + OH - 1) / OH); }
+    static cudaError_t setup(FieldArgs<float> &A, int sms)
     {
         A.ahead = sms * MINB;
-        cudaError_t e = cudaFuncSetAttribute(field_tile_kernel<T, BW, BH, P, NS, MINB, true>,
+        cudaError_t e = cudaFuncSetAttribute(field_tile_kernel<BW, BH, P, NS, MINB, true>,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        return e ? e : cudaFuncSetAttribute(field_tile_kernel<T, BW, BH, P, NS, MINB, false>,
+        return e ? e : cudaFuncSetAttribute(field_tile_kernel<BW, BH, P, NS, MINB, false>,
                                             cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     }
-    static void launch(const FieldArgs<T> &A, bool first, cudaStream_t s)
+    static void launch(const FieldArgs<float> &A, bool first, cudaStream_t s)
     {
         if (first)
-            field_tile_kernel<T, BW, BH, P, NS, MINB, true><<<grid(A), threads, smem, s>>>(A);
+            field_tile_kernel<BW, BH, P, NS, MINB, true><<<grid(A), threads, smem, s>>>(A);
         else
-            field_tile_kernel<T, BW, BH, P, NS, MINB, false><<<grid(A), threads, smem, s>>>(A);
+            field_tile_kernel<BW, BH, P, NS, MINB, false><<<grid(A), threads, smem, s>>>(A);
     }
 };
 
@@ -451,10 +539,10 @@ struct Strips {
 // by launches of the shape SH: the rows outside are left as they are and feed
 // the range's edge rows.  Y: nullptr, or every stage's own output arrays
 // (SH::stages == 1; X is then not written).  Without correctors the step is
-// the forward-Euler predictor alone, undamped.
+// the forward-Euler predictor alone, undamped.  lead: FieldArgs.
 template <typename T, typename SH>
 cudaError_t run_field(grpic_ctx *ctx, T *const X[6], T *const J[3], int64_t ld, const T *tab, const T *col1d,
-                      cudaStream_t s, int j_lo, int j_hi, T *const *Y = nullptr)
+                      cudaStream_t s, int j_lo, int j_hi, T *const *Y = nullptr, bool lead = false)
 {
     const int N = ctx->prm.n_field_iter;
     FieldArgs<T> A;
@@ -465,7 +553,9 @@ cudaError_t run_field(grpic_ctx *ctx, T *const X[6], T *const J[3], int64_t ld, 
     A.slab = ctx->slab;
     A.dt = (T)ctx->prm.dt;
     A.as = (T)(1.0 - ctx->prm.beta_field);
+    A.bs = (T)ctx->prm.beta_field;
     A.dtbs = (T)(ctx->prm.dt * ctx->prm.beta_field);
+    A.lead = lead;
     A.dth = (T)ctx->g.dth;
     A.tab = tab;
     A.col1d = col1d;
@@ -474,21 +564,35 @@ cudaError_t run_field(grpic_ctx *ctx, T *const X[6], T *const J[3], int64_t ld, 
     A.rows = 0;
     for (int k = 0; k < 3; ++k) A.J[k] = J[k];
     const int launches = (N + SH::stages) / SH::stages;
+    // A launch's halo reads the iterate at other CTAs' points, so it writes other
+    // arrays.  Tiles: the iterate alternates between a buffer and, X^n being copied
+    // by the first launch, the caller's arrays; strips: between two buffers, the
+    // last stage writing the caller's (of X^n each thread reads its own point).
+    constexpr bool tiles = SH::stages > 1;
+    const bool in_buffer = !Y && (tiles ? launches % 2 == 1 : launches == 1);  // the result
     cudaError_t e = SH::setup(A, sm_count(ctx->device));
     for (int l = 0; l < launches && e == cudaSuccess; ++l) {
         const bool last = l == launches - 1;
         A.last = last && N > 0;
         A.ns = std::min(SH::stages, N + 1 - l * SH::stages);
         for (int k = 0; k < 6; ++k) {
+            T *const buf[2] = {fslot<T>(ctx, 6 + k, ld), fslot<T>(ctx, 12 + k, ld)};
             A.Bs[k] = fslot<T>(ctx, k, ld);
-            A.Xi[k] = l == 0 ? X[k] : (Y ? Y[6 * (l - 1) + k] : fslot<T>(ctx, 6 + 6 * ((l - 1) & 1) + k, ld));
-            // (a single launch's halo reads X^n of other CTAs' points: it writes a buffer)
-            A.Xo[k] = Y ? Y[6 * l + k] : (last && l > 0 ? X[k] : fslot<T>(ctx, 6 + 6 * (l & 1) + k, ld));
+            if (tiles) {
+                A.Xi[k] = l % 2 ? buf[0] : X[k];
+                A.Xo[k] = l % 2 ? X[k] : buf[0];
+                A.Xn[k] = buf[1];
+                A.Xs[k] = launches > 1 ? buf[1] : nullptr;
+            } else {
+                A.Xi[k] = l == 0 ? X[k] : (Y ? Y[6 * (l - 1) + k] : buf[(l - 1) & 1]);
+                A.Xo[k] = Y ? Y[6 * l + k] : (last && l > 0 ? X[k] : buf[l & 1]);
+                A.Xn[k] = X[k];
+            }
         }
         SH::launch(A, l == 0, s);
         e = cudaGetLastError();
     }
-    if (launches == 1 && !Y)
+    if (in_buffer)
         for (int k = 0; k < 6 && e == cudaSuccess; ++k) {
             const int hi = std::min(j_hi, ctx->g.nth + (half_t(k) ? 0 : 1));
             if (hi > j_lo)
@@ -501,9 +605,9 @@ cudaError_t run_field(grpic_ctx *ctx, T *const X[6], T *const J[3], int64_t ld, 
 
 using Strips64 = Strips<double, 64, 4, 2>;
 using Narrow64 = Strips<double, 32, 8, 2>;
-using Strips32 = Strips<float, 64, 4, 4>;
-using Wide32 = Tiles<float, 64, 24, 3, 4, 1>;
-using Small32 = Tiles<float, 32, 16, 1, 4, 2>;
+using Strips32 = Strips<float, 64, 4, 3>;
+using Wide32 = Tiles<64, 24, 3, 4, 1>;
+using Small32 = Tiles<32, 16, 1, 4, 2>;
 
 cudaError_t run_field64(grpic_ctx *ctx, double *const X[6], double *const J[3], int64_t ld, cudaStream_t s, int j_lo,
                         int j_hi, double *const *Y = nullptr)
@@ -552,16 +656,26 @@ cudaError_t launch_field64(grpic_ctx *ctx, grpic_fields *f, cudaStream_t s, int 
 // (grpic_set_field_path); the same operations per point either way.  Of the
 // two tiles the wide one has the smaller halo; the small one is taken while
 // the wide one's CTAs do not fill the SMs.
+// Which product of the corrector's sum is inside the fused multiply-add
+// (FieldArgs::lead) goes by the arrays: beta_s C on the whole grid with 16-byte
+// rows and bases, alpha_s C^n elsewhere.  Both are equally good; these are the
+// orders that runs on such arrays have always had, so a run that is continued or
+// repeated keeps its bits.
 cudaError_t launch_field32(grpic_ctx *ctx, grpic_fields *f, cudaStream_t s, int j_lo, int j_hi)
 {
     const int rows = ctx->g.nth + 1, sms = sm_count(ctx->device);
     if (j_hi < 0) j_hi = rows;
     const FieldPtrs<float> P(f);
-    if (!(ctx->field_fused && j_lo == 0 && j_hi == rows))
-        return run_field<float, Strips32>(ctx, P.X, P.J, f->ld, ctx->tab32, ctx->col1d32, s, j_lo, j_hi);
+    const bool whole = j_lo == 0 && j_hi == rows;
+    bool lead = whole && f->ld % 4 == 0;
+    for (int k = 0; k < 6; ++k) lead = lead && (uintptr_t)P.X[k] % 16 == 0;
+    if (!(ctx->field_fused && whole))
+        return run_field<float, Strips32>(ctx, P.X, P.J, f->ld, ctx->tab32, ctx->col1d32, s, j_lo, j_hi, nullptr, lead);
     const int64_t wide = (int64_t)((ctx->g.ld_tab + Wide32::OW - 1) / Wide32::OW) * ((rows + Wide32::OH - 1) / Wide32::OH);
-    return wide <= sms ? run_field<float, Small32>(ctx, P.X, P.J, f->ld, ctx->tab32, ctx->col1d32, s, j_lo, j_hi)
-                       : run_field<float, Wide32>(ctx, P.X, P.J, f->ld, ctx->tab32, ctx->col1d32, s, j_lo, j_hi);
+    return wide <= sms ? run_field<float, Small32>(ctx, P.X, P.J, f->ld, ctx->tab32, ctx->col1d32, s, j_lo, j_hi, nullptr,
+                                                   lead)
+                       : run_field<float, Wide32>(ctx, P.X, P.J, f->ld, ctx->tab32, ctx->col1d32, s, j_lo, j_hi, nullptr,
+                                                  lead);
 }
 
 }  // namespace grpic
