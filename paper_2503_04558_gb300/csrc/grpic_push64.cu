@@ -310,11 +310,13 @@ __device__ __forceinline__ void sincos_row(const GridDev &g, int j, double f, do
 
 // FP32 view of 1 + gamma^ij u_i u_j, a few 1e-6 of its terms off: whether the
 // FIDO Lorentz factor can reach `thr` (the FP64 decision is taken only then; a
-// margin of 2 % in the square covers the cancellation between the terms)
-__device__ __forceinline__ bool may_reach(float a, float r, float th, double u0, double u1, double u2, float thr2)
+// margin of 2 % in the square covers the cancellation between the terms).  The
+// angle is taken from the nearer pole before it is cut to FP32: pi - theta, for
+// theta close to pi, has no relative precision left in a float theta.
+__device__ __forceinline__ bool may_reach(float a, float r, double th, double u0, double u1, double u2, float thr2)
 {
-    float s, c;
-    sincosf(th, &s, &c);
+    float s, c;  // (cos enters by its square)
+    sincosf((float)(__double2hiint(th) >= 0x3ff921fb ? M_PI - th : th), &s, &c);
     const float v0 = (float)u0, v1 = (float)u1, v2 = (float)u2;
     const float ir = 1.0f / fmaf(a * c, a * c, r * r), z = 2.0f * r * ir;
     const float t0 = (fmaf(a, a, r * r) * ir - z / (1.0f + z)) * v0 * v0, t1 = 2.0f * a * ir * v0 * v2;
@@ -521,7 +523,7 @@ __global__ void __launch_bounds__(PUSH64_T, 512 / PUSH64_T) push64_kernel(Push64
                     // which then skip the metric: the same decision)
                     const bool charged = A.massive[sp] && A.qm[sp] != 0.0;
                     const bool drawn = !A.massive[sp] && uniform53(A.seed, (uint64_t)p, A.step, 1) < A.pconv;
-                    if (drawn || (charged && may_reach((float)g.a, (float)r, (float)th, u[0], u[1], u[2],
+                    if (drawn || (charged && may_reach((float)g.a, (float)r, th, u[0], u[1], u[2],
                                                        A.gthr2f))) {
                         KS m;
                         ks_point(g.a, r, th, m);
