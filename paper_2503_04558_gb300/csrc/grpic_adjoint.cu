@@ -1160,13 +1160,17 @@ extern "C" grpic_status grpic_horizon_flux(grpic_ctx *ctx, const grpic_fields *f
         hp[3 + k] = (double *)f->B[k];
     }
     FAdj A{ctx->g.nr, ctx->g.nth, f->ld, ctx->g.ld_tab, ctx->slab, ctx->tab, ctx->col1d};
-    double *dev = (double *)((char *)ctx->d_status + 48);  // behind the status word and the charges
+    // the call's own word: calls on one context from several streams or threads
+    // do not meet
+    double *dev = nullptr;
+    if (cudaMalloc(&dev, sizeof(double)) != cudaSuccess) return GRPIC_ENOMEM;
     cudaMemsetAsync(dev, 0, sizeof(double), s);
     flux_kernel<<<1, 256, 0, s>>>(A, six(hp), i_horizon, ctx->g.dth, 1.0, dev);
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaMemcpyAsync(out, dev, sizeof(double), cudaMemcpyDeviceToHost, s);
-    cudaStreamSynchronize(s);
-    return e == cudaSuccess ? GRPIC_OK : GRPIC_ECUDA;
+    const cudaError_t es = cudaStreamSynchronize(s);
+    cudaFree(dev);
+    return e == cudaSuccess && es == cudaSuccess ? GRPIC_OK : GRPIC_ECUDA;
 }
 
 // What the spin derivative of one field update needs: the derivative
