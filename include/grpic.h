@@ -352,8 +352,9 @@ grpic_status grpic_adjoint_field_step(grpic_ctx *ctx, const grpic_fields *lam_in
  * and step).  The last segment is recorded during the forward pass itself, so
  * checkpoint_every >= nsteps trades that memory for no recomputation at all.
  * The memory is one block; it stays with the context for the next call while
- * it is at most a sixteenth of the device's (freed by grpic_destroy, or when a
- * later call needs more), and is freed before the call returns otherwise.
+ * it is at most a sixteenth of the device's (freed by grpic_destroy, when a
+ * later gradient needs more, or when another call on the context would fail for
+ * want of memory), and is freed before the call returns otherwise.
  *   p0:  n live or dead particles (FP64 SoA r, theta, u_r, u_theta, u_phi,
  *        tag); not modified.  p0->d_count is ignored (p0->n is used).
  *   f0:  the fields at step 0 (D, B; f0->J unused); not modified.

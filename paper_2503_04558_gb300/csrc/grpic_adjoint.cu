@@ -1227,7 +1227,7 @@ extern "C" grpic_status grpic_adjoint_field_step(grpic_ctx *ctx, const grpic_fie
     int64_t ld = lam_in->ld;
     size_t fn = (size_t)(ctx->g.nth + 1) * ld;
     double *base = nullptr;
-    if (cudaMalloc(&base, 18 * fn * sizeof(double)) != cudaSuccess) return GRPIC_ENOMEM;
+    if (ctx_malloc(ctx, &base, 18 * fn * sizeof(double)) != cudaSuccess) return GRPIC_ENOMEM;
     double *work[18], *in[6], *out[6], *J[3];
     for (int k = 0; k < 18; ++k) work[k] = base + k * fn;
     for (int k = 0; k < 3; ++k) {
@@ -1329,10 +1329,13 @@ extern "C" grpic_status grpic_adjoint_grad(grpic_ctx *ctx, const grpic_particles
         for (auto &q : Ystage) q = place(fn * sizeof(double));
     };
     layout();
+    // (the context's own scratch first: it may take the kept block's memory)
+    if (ensure_field_scratch_ext(ctx, ld) != GRPIC_OK || ensure_particle_scratch_ext(ctx, np) != GRPIC_OK)
+        return GRPIC_ENOMEM;
     // The block stays with the context for the next gradient while it is at most a
     // sixteenth of the device's memory (mapping 5.5 GB and unmapping it took 27 of
-    // 98 ms); a larger one is given back at once, the kept one by grpic_destroy or
-    // when a call needs more.
+    // 98 ms); a larger one is given back at once, the kept one by grpic_destroy, when
+    // a gradient needs more, or when another call of the context finds no memory.
     if (ctx->adj_bytes < need) {
         cudaFree(ctx->adj_block);
         ctx->adj_block = nullptr;
@@ -1415,10 +1418,6 @@ extern "C" grpic_status grpic_adjoint_grad(grpic_ctx *ctx, const grpic_particles
         return r;
     };
     // ---- forward with checkpoints --------------------------------------
-    if (ensure_field_scratch_ext(ctx, ld) != GRPIC_OK || ensure_particle_scratch_ext(ctx, np) != GRPIC_OK) {
-        cleanup();
-        return GRPIC_ENOMEM;
-    }
     // the last segment, the first the reverse sweep needs, is recorded here
     // (its states, the push's record and, for the spin derivative, its
     // currents) instead of being recomputed from a checkpoint

@@ -70,7 +70,7 @@ extern "C" grpic_status grpic_adjoint_spin(grpic_ctx *ctx, const grpic_particles
     std::vector<void *> allocs;
     auto dalloc = [&](size_t bytes) -> void * {
         void *q = nullptr;
-        if (cudaMalloc(&q, bytes) != cudaSuccess) return nullptr;
+        if (ctx_malloc(ctx, &q, bytes) != cudaSuccess) return nullptr;
         allocs.push_back(q);
         return q;
     };

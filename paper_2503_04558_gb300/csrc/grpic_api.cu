@@ -141,8 +141,8 @@ grpic_status ensure_field_scratch(grpic_ctx *ctx, int64_t ld)
     if (ctx->q32) cudaFree(ctx->q32);
     ctx->fscratch = ctx->q32 = nullptr;
     ctx->fscratch_ld = 0;
-    cudaError_t e = cudaMalloc(&ctx->fscratch, need);
-    if (e == cudaSuccess && qneed) e = cudaMalloc(&ctx->q32, qneed);
+    cudaError_t e = ctx_malloc(ctx, &ctx->fscratch, need);
+    if (e == cudaSuccess && qneed) e = ctx_malloc(ctx, &ctx->q32, qneed);
     if (e != cudaSuccess) {
         if (ctx->fscratch) cudaFree(ctx->fscratch);
         ctx->fscratch = ctx->q32 = nullptr;
@@ -179,8 +179,8 @@ grpic_status ensure_particle_scratch(grpic_ctx *ctx, int64_t n)
     ctx->d_keys = nullptr;
     ctx->d_perm = nullptr;
     ctx->keys_cap = 0;
-    if (cudaMalloc(&ctx->d_keys, sizeof(int32_t) * (size_t)n) != cudaSuccess ||
-        cudaMalloc(&ctx->d_perm, sizeof(int32_t) * (size_t)n) != cudaSuccess)
+    if (ctx_malloc(ctx, &ctx->d_keys, sizeof(int32_t) * (size_t)n) != cudaSuccess ||
+        ctx_malloc(ctx, &ctx->d_perm, sizeof(int32_t) * (size_t)n) != cudaSuccess)
         return fail(ctx, GRPIC_ENOMEM, "particle scratch allocation failed");
     ctx->keys_cap = n;
     ctx->perm_cap = n;
@@ -955,9 +955,9 @@ grpic_status grpic_charge_check(grpic_ctx *ctx, const grpic_particles *p, const 
     const size_t n = (size_t)(ctx->g.nth + 1) * f->ld;
     double *rho = nullptr, *divD = nullptr;
     unsigned long long *dout = nullptr;
-    cudaError_t e = cudaMalloc(&rho, n * sizeof(double));
-    if (e == cudaSuccess) e = cudaMalloc(&divD, n * sizeof(double));
-    if (e == cudaSuccess) e = cudaMalloc(&dout, 2 * sizeof(unsigned long long));
+    cudaError_t e = ctx_malloc(ctx, &rho, n * sizeof(double));
+    if (e == cudaSuccess) e = ctx_malloc(ctx, &divD, n * sizeof(double));
+    if (e == cudaSuccess) e = ctx_malloc(ctx, &dout, 2 * sizeof(unsigned long long));
     if (e == cudaSuccess) e = launch_charge_check(ctx, p, f, rho, divD, base, state, dout, S(stream));
     unsigned long long h[2] = {0, 0};
     if (e == cudaSuccess) e = cudaMemcpyAsync(h, dout, sizeof h, cudaMemcpyDeviceToHost, S(stream));

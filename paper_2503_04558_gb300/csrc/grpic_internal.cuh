@@ -306,6 +306,21 @@ inline int sm_count(int device)
     cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, device);
     return n;
 }
+// device memory for a context's call: where there is none left, the gradient's kept
+// block (adj_block) is given back first.  Not while a gradient runs in it.
+template <typename T>
+inline cudaError_t ctx_malloc(grpic_ctx *ctx, T **p, size_t bytes)
+{
+    cudaError_t e = cudaMalloc(p, bytes);
+    if (e == cudaErrorMemoryAllocation && ctx->adj_block) {
+        cudaGetLastError();
+        cudaFree(ctx->adj_block);
+        ctx->adj_block = nullptr;
+        ctx->adj_bytes = 0;
+        e = cudaMalloc(p, bytes);
+    }
+    return e;
+}
 cudaError_t launch_tables(grpic_ctx *ctx, cudaStream_t s);
 cudaError_t launch_init_fields(grpic_ctx *ctx, int kind, double B0, const grpic_fields *f, cudaStream_t s);
 // push (fused with the deposit) of the particles of `in` into `p`: in place

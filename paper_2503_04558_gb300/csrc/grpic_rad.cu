@@ -299,10 +299,10 @@ cudaError_t ensure_rad_scratch(grpic_ctx *ctx, int64_t cap)
     ctx->d_spawn = nullptr;
     ctx->d_rad = nullptr;
     const int64_t nbp = (cap + RB - 1) / RB, nbc = (ncell + RB - 1) / RB;
-    cudaError_t e = cudaMalloc(&ctx->d_spawn, sizeof(int32_t) * (size_t)cap);
+    cudaError_t e = ctx_malloc(ctx, &ctx->d_spawn, sizeof(int32_t) * (size_t)cap);
     // rad: [block sums / offsets of slots: nbp + 1] [of cells: nbc + 1] [charged per cell: ncell] [flags: ncell]
     if (e == cudaSuccess)
-        e = cudaMalloc(&ctx->d_rad, sizeof(int32_t) * (size_t)(2 * (nbp + 1) + 2 * (nbc + 1) + 2 * ncell));
+        e = ctx_malloc(ctx, &ctx->d_rad, sizeof(int32_t) * (size_t)(2 * (nbp + 1) + 2 * (nbc + 1) + 2 * ncell));
     ctx->rad_cap = e == cudaSuccess ? cap : 0;
     return e;
 }
