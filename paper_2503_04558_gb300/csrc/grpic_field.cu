@@ -70,6 +70,7 @@ struct FieldArgs {
     int ns;          // tile kernel: stages of this launch
     int ahead;       // tile kernel: CTAs running at a time
     int last;        // the last stage is damped
+    int carry;       // strip kernel: copy the rows next to the range to the next iterate
 };
 
 __host__ __device__ constexpr bool half_r(int k) { return k == 0 || k == 4 || k == 5; }
@@ -425,6 +426,12 @@ __global__ void __launch_bounds__(BW *RT, RES) field_strip_kernel(const __grid_c
             B[k] = on ? __ldg((FIRST ? A.Xi[k] : A.Bs[k]) + q) : T(0);  // X^n or what the predictor left
             if (sizeof(T) == 4 && !FIRST) XN[k] = on ? __ldg(A.Xn[k] + q) : T(0);
         }
+        if (A.carry && (j == A.j_lo - 1 || j == A.j_hi) && j <= jb && j >= 0 && j <= nth && col_in && bc >= 1 &&
+            bc <= BW - 2) {
+#pragma unroll
+            for (int k = 0; k < 6; ++k)
+                if (!(half_t(k) && j == nth)) A.Xo[k][(size_t)j * A.ld + c] = X[k];
+        }
         products(K, X, S, NP, (int)threadIdx.x);
         __syncthreads();
         auxiliary(K, X, S, NP, el, er, E, NE, ((j + 1) & (RING - 1)) * BW + bc);
@@ -537,7 +544,8 @@ struct Strips {
 
 // The update of rows [j_lo, j_hi) of X (D, then B; in place) with currents J
 // by launches of the shape SH: the rows outside are left as they are and feed
-// the range's edge rows.  Y: nullptr, or every stage's own output arrays
+// the range's edge rows in every stage (their two neighbours go along with the
+// iterates).  Y: nullptr, or every stage's own output arrays
 // (SH::stages == 1; X is then not written).  Without correctors the step is
 // the forward-Euler predictor alone, undamped.  lead: FieldArgs.
 template <typename T, typename SH>
@@ -562,6 +570,7 @@ cudaError_t run_field(grpic_ctx *ctx, T *const X[6], T *const J[3], int64_t ld, 
     A.j_lo = j_lo;
     A.j_hi = j_hi;
     A.rows = 0;
+    const bool whole = j_lo == 0 && j_hi == ctx->g.nth + 1;
     for (int k = 0; k < 3; ++k) A.J[k] = J[k];
     const int launches = (N + SH::stages) / SH::stages;
     // A launch's halo reads the iterate at other CTAs' points, so it writes other
@@ -574,6 +583,7 @@ cudaError_t run_field(grpic_ctx *ctx, T *const X[6], T *const J[3], int64_t ld, 
     for (int l = 0; l < launches && e == cudaSuccess; ++l) {
         const bool last = l == launches - 1;
         A.last = last && N > 0;
+        A.carry = !tiles && !whole && !last;
         A.ns = std::min(SH::stages, N + 1 - l * SH::stages);
         for (int k = 0; k < 6; ++k) {
             T *const buf[2] = {fslot<T>(ctx, 6 + k, ld), fslot<T>(ctx, 12 + k, ld)};
