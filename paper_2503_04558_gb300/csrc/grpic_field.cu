@@ -28,12 +28,13 @@ namespace {
 // fields E_i, H_i themselves (auxiliary()), then the circulations (circulation()),
 // so no table value of a neighbour is read.
 //
-// FP64: the predictor leaves the part of the correctors that does not change,
-// the base
-//   X^n + dt (alpha_s C(X^n) - J / A),
-// and a corrector is base + (dt beta_s / A) circ(X): X^n, C^n and J are not read
-// again.  52 operations per point and stage (122 when each point evaluated its
-// neighbours' auxiliary fields and combined X^n, C^n and J in every stage).
+// FP64: the predictor leaves the part of a corrector's circulation that does not
+// change, alpha_s circ(X^n) - J, and a corrector is
+//   X^n + (dt / A) (beta_s circ(X) + that),
+// one rounding of X's size per stage.  56 operations per point and stage (122 when
+// each point evaluated its neighbours' auxiliary fields and combined X^n, C^n and J
+// in every stage; 52 with X^n folded in too, whose second rounding left B^r 1.4
+// times further from 64 bits' value at 128^2).
 //
 // FP32: the order of the roundings is fixed, operation by operation:
 //   products t x of a pair: fma(own t, own x, round(neighbour's t x)), halved;
@@ -48,20 +49,20 @@ namespace {
 // every launch shape, and the same as before the shapes were changed.  (Folding
 // alpha_s, J and dt / A into a base as in FP64: 0.63 ms an update at 2048^2, but two
 // steps at that size then ended with J^phi 2.4e-4 off.)
-// One update (8 stages): FP32 2048^2 1.29 -> 0.81 ms, FP64 1024^2 2.44 -> 1.15
-// ms (82 % of the FP64 pipe's cycles); FP64 128^2 0.128 -> 0.066 ms.
+// One update (8 stages): FP32 2048^2 1.29 -> 0.81 ms, FP64 1024^2 2.44 -> 1.21
+// ms; FP64 128^2 0.128 -> 0.066 ms.
 template <typename T>
 struct FieldArgs {
     int nr, nth, ldt, ld;
     size_t slab;
-    T dt, as, bs, dtbs, dth;
+    T dt, as, bs, dth;
     const T *tab;
     const T *col1d;  // dr_prim, dr_dual, damp_int, damp_half
     const T *Xi[6];  // the iterate at the launch's first stage
     T *Xo[6];        // the iterate after its last one
-    T *Bs[6];        // FP64: the base; FP32: C^n, times alpha_s if `lead` (written by the
-                     // first launch, read by the others)
-    const T *Xn[6];  // FP32: X^n for the launches after the first
+    T *Bs[6];        // FP64: alpha_s circ(X^n) - J; FP32: C^n, times alpha_s if `lead`
+                     // (written by the first launch, read by the others)
+    const T *Xn[6];  // X^n for the launches after the first
     T *Xs[6];        // FP32 tiles: a copy of X^n, written by the first launch
     const T *J[3];
     int lead;        // FP32: fma(beta_s, C, alpha_s C^n), else fma(alpha_s, C^n, beta_s C)
@@ -183,13 +184,24 @@ __device__ __forceinline__ float correct(float C, float W, float Q, float Xn, fl
     return fmaf(-Jd, A.dt, fmaf(A.dt, m, Xn));
 }
 
-// FP64: the predictor at one component: X^n -> X~ and the base B
-template <typename T>
-__device__ __forceinline__ void predict(T C, T W, T J, T dt, T as, T &X, T &B)
+// FP64: the predictor at one component, X^n -> X~; Q: alpha_s circ^n - J, what the
+// correctors add to beta_s circ
+__device__ __forceinline__ void predict(double C, double W, double J, const FieldArgs<double> &A, double &X, double &Q)
 {
-    const T Cn = C * W;
-    B = fmat(dt, fmat(as, Cn, -(J * W)), X);
-    X = fmat(dt, fmat(-J, W, Cn), X);
+    Q = fma(A.as, C, -J);
+    X = fma(C - J, A.dt * W, X);
+}
+// ... and beta_s circ + Q of a corrector (bd, bp, br: beta_s times dth, drp, drd)
+__device__ __forceinline__ void circulation_on(const double *E, int m, int o, int l, int r, int d, int u, double bs,
+                                               double bd, double bp, double br, const double *Q, double *C)
+{
+    const double hp = E[2 * m + o], ep = E[5 * m + o];
+    C[0] = fma(bs, hp - E[2 * m + d], Q[0]);
+    C[1] = fma(bs, E[2 * m + l] - hp, Q[1]);
+    C[2] = fma(E[m + o] - E[m + l], bd, fma(E[d] - E[o], br, Q[2]));
+    C[3] = fma(bs, ep - E[5 * m + u], Q[3]);
+    C[4] = fma(bs, E[5 * m + r] - ep, Q[4]);
+    C[5] = fma(E[4 * m + o] - E[4 * m + r], bd, fma(E[3 * m + u] - E[3 * m + o], bp, Q[5]));
 }
 
 // one component's new value at (i, j) with the guard copies of the first and
@@ -424,7 +436,6 @@ __global__ void __launch_bounds__(BW *RT, RES) field_strip_kernel(const __grid_c
             const bool on = upd && !(half_r(k) && !ph_h) && !(half_t(k) && ju == nth) && !((k == 2 || k == 4) && axis);
             W[k] = on ? __ldg(A.tab + inv_area(k) * A.slab + (unsigned)(ju * A.ldt + c)) : T(0);
             B[k] = on ? __ldg((FIRST ? A.Xi[k] : A.Bs[k]) + q) : T(0);  // X^n or what the predictor left
-            if (sizeof(T) == 4 && !FIRST) XN[k] = on ? __ldg(A.Xn[k] + q) : T(0);
         }
         if (A.carry && (j == A.j_lo - 1 || j == A.j_hi) && j <= jb && j >= 0 && j <= nth && col_in && bc >= 1 &&
             bc <= BW - 2) {
@@ -436,12 +447,22 @@ __global__ void __launch_bounds__(BW *RT, RES) field_strip_kernel(const __grid_c
         __syncthreads();
         auxiliary(K, X, S, NP, el, er, E, NE, ((j + 1) & (RING - 1)) * BW + bc);
         load(j + RT);
+        // (X^n here, where the coefficients' registers are free, not with W and B: FP64
+        // 512^2 0.46 -> 0.40 ms)
+#pragma unroll
+        for (int k = 0; k < 6; ++k) {
+            const bool on = upd && !(half_r(k) && !ph_h) && !(half_t(k) && ju == nth) && !((k == 2 || k == 4) && axis);
+            if (!FIRST) XN[k] = on ? __ldg(A.Xn[k] + q) : T(0);
+        }
         __syncthreads();
         if (upd) {
             const int o = (j & (RING - 1)) * BW + bc;
+            const int d = (ju & (RING - 1)) * BW + bc, u = ((j + 1) & (RING - 1)) * BW + bc;
             T C[6];
-            circulation(E, NE, o, o - 1, o + 1, (ju & (RING - 1)) * BW + bc, ((j + 1) & (RING - 1)) * BW + bc, A.dth,
-                        drp, drd, C);
+            if constexpr (FIRST || sizeof(T) == 4)
+                circulation(E, NE, o, o - 1, o + 1, d, u, A.dth, drp, drd, C);
+            else
+                circulation_on(E, NE, o, o - 1, o + 1, d, u, A.bs, A.bs * A.dth, A.bs * drp, A.bs * drd, B, C);
             const size_t row = (size_t)ju * A.ld;
 #pragma unroll
             for (int k = 0; k < 6; ++k) {
@@ -455,13 +476,15 @@ __global__ void __launch_bounds__(BW *RT, RES) field_strip_kernel(const __grid_c
                         float jd;
                         predict(C[k], W[k], J, A, v, b, jd);
                     } else {
-                        predict(C[k], W[k], J, A.dt, A.as, v, b);
+                        predict(C[k], W[k], J, A, v, b);
                     }
                     if ((k == 2 || k == 4) && axis) v = b = T(0);
-                } else if constexpr (sizeof(T) == 4) {
-                    v = (k == 2 || k == 4) && axis ? 0.0f : correct(C[k], W[k], B[k], XN[k], __fmul_rn(J, W[k]), A);
                 } else {
-                    v = fmat(C[k], W[k] * A.dtbs, B[k]);
+                    if constexpr (sizeof(T) == 4)
+                        v = correct(C[k], W[k], B[k], XN[k], __fmul_rn(J, W[k]), A);
+                    else
+                        v = fma(C[k], A.dt * W[k], XN[k]);
+                    if ((k == 2 || k == 4) && axis) v = T(0);
                 }
                 if (A.last) v *= half_r(k) ? dmh : dmi;
                 put_value(A.Xo[k] + row, c, i, half_r(k) ? nr - 1 : nr, A.ldt, v);
@@ -503,7 +526,8 @@ struct Tiles {
 
 // A launch shape of the strip kernel.  The rows per CTA are those for which the
 // fullest SM has the least to do: each of its CTAs forms the auxiliary fields of
-// rows + 2 rows (28 operations a point) and updates `rows` of them (24), in
+// rows + 2 rows (28 operations a point) and updates `rows` of them (28; the rule
+// takes 24, which measured the same or better), in
 // (rows + 2) / RT rounds whose latency (about ROUND operations' time) CTAs
 // resident together hide from each other.  So long strips on large grids (few
 // halo rows) and one short round, spread over all SMs, on small ones.
@@ -562,7 +586,6 @@ cudaError_t run_field(grpic_ctx *ctx, T *const X[6], T *const J[3], int64_t ld, 
     A.dt = (T)ctx->prm.dt;
     A.as = (T)(1.0 - ctx->prm.beta_field);
     A.bs = (T)ctx->prm.beta_field;
-    A.dtbs = (T)(ctx->prm.dt * ctx->prm.beta_field);
     A.lead = lead;
     A.dth = (T)ctx->g.dth;
     A.tab = tab;
