@@ -33,8 +33,8 @@
 // the precondition holds by construction and only 7 and 8 are launched.  Elsewhere
 // a count pass checks it (every key a neighbour of its segment, live count = the
 // previous sort's) and raises a device flag when it fails; the general kernels then
-// run instead.  Every kernel of both paths reads the flag and strides over its work
-// with a fixed grid, so the path not taken costs one flag read per block.
+// run instead: there every kernel of both paths reads the flag and strides over its
+// work with a fixed grid, so the path not taken costs one flag read per block.
 #include "grpic_internal.cuh"
 
 #include <algorithm>
@@ -718,7 +718,8 @@ __device__ __forceinline__ int first_slot(const int32_t *cnt9, const int32_t *of
 // launch, and 72 B a cell written and read.)
 __global__ void __launch_bounds__(256, 8) neighbour_perm_kernel(const int32_t *off_old, const int32_t *off_new,
                                                              const int32_t *cnt9, const int32_t *keys, int nr, int nth,
-                                                             int per, int64_t nmax, int32_t *perm, const int32_t *flag)
+                                                             int per, int64_t nmax, int32_t *perm, const int32_t *flag,
+                                                             int *status)
 {
     if (flag && *flag) return;
     __shared__ int run_sh[8][TASK_CELLS * 9];
@@ -763,13 +764,16 @@ __global__ void __launch_bounds__(256, 8) neighbour_perm_kernel(const int32_t *o
                 // the precondition holds here (checked by the count pass, or
                 // by construction when the push counted: moves of at most one
                 // cell), so the direction follows from k - s alone; a key out
-                // of the 9 (never seen) is dropped rather than indexing run[]
+                // of the 9 (never seen) is reported rather than indexing run[]
                 int key2 = -1;
                 if (p < end && (unsigned)k < (unsigned)ncell) {
                     const int delta = k - (int)(s0 + c);
                     const int dj = (delta > 1) - (delta < -1);
                     const int di = delta - dj * nr;
-                    if ((unsigned)(di + 1) <= 2u) key2 = c * 9 + (dj + 1) * 3 + (di + 1);
+                    if ((unsigned)(di + 1) <= 2u)
+                        key2 = c * 9 + (dj + 1) * 3 + (di + 1);
+                    else
+                        set_status(status, GRPIC_ERANGE);
                 }
                 const unsigned peers = __match_any_sync(FULL, key2);
                 const bool has = key2 >= 0;
@@ -935,7 +939,8 @@ cudaError_t launch_sort_step(grpic_ctx *ctx, grpic_particles *p, grpic_particles
         }
         if (p->n > 0)
             neighbour_perm_kernel<<<grid, 256, 0, s>>>(ctx->d_offset_prev, ctx->d_offset, ctx->d_cnt9, ctx->d_keys,
-                                                       ctx->g.nr, ctx->g.nth, per, p->n, ctx->d_perm, nullptr);
+                                                       ctx->g.nr, ctx->g.nth, per, p->n, ctx->d_perm, nullptr,
+                                                       ctx->d_status);
         if (p->n > 0 && materialize) launch_gather(ctx, p, q, gp, s);
         return cudaGetLastError();
     }
@@ -959,7 +964,7 @@ cudaError_t launch_sort_step(grpic_ctx *ctx, grpic_particles *p, grpic_particles
     add_back<<<(unsigned)((nscan + 255) / 256), 256, 0, s>>>(ctx->d_offset, ctx->d_blocksum, nscan);
     if (neighbour && p->n > 0)
         neighbour_perm_kernel<<<grid, 256, 0, s>>>(ctx->d_offset_prev, ctx->d_offset, ctx->d_cnt9, ctx->d_keys,
-                                                   ctx->g.nr, ctx->g.nth, per, p->n, ctx->d_perm, flag);
+                                                   ctx->g.nr, ctx->g.nth, per, p->n, ctx->d_perm, flag, ctx->d_status);
     // general path to the permutation (skipped on the device when the neighbour sort applied)
     int32_t *nbig = ctx->d_cursor + nscan;
     cudaMemsetAsync(ctx->d_cursor, 0, sizeof(int32_t) * (nscan + 1), s);  // with the count behind the cursors
