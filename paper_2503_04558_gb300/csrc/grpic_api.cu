@@ -132,8 +132,9 @@ size_t fsize(const grpic_ctx *ctx) { return ctx->prm.precision == 64 ? sizeof(do
 grpic_status ensure_field_scratch(grpic_ctx *ctx, int64_t ld)
 {
     static_assert(sizeof(int64_t) == 8, "");
-    // 18 arrays: C^n (6) and two iterate buffers (12), stride ld; in the
-    // FP32 form also the push's stencil quads of the six components
+    // 18 arrays: what the field update's predictor leaves for the correctors (6)
+    // and two iterate buffers, or one and X^n (12), stride ld; in the FP32 form
+    // also the push's stencil quads of the six components
     size_t need = 18 * (size_t)(ctx->g.nth + 1) * (size_t)ld * fsize(ctx);
     size_t qneed = ctx->prm.precision == 32 ? 6 * (size_t)(ctx->g.nth + 1) * (size_t)ld * 16 : 0;
     if (ctx->fscratch && ctx->fscratch_ld == ld) return GRPIC_OK;

@@ -223,12 +223,16 @@ __device__ __forceinline__ int row_of(const GridDev &g, double x2)
 }
 
 // Column of r > 0 and the offset in it (0 <= f < 1); columns more than NG beyond
-// the grid are reported with an offset of 1/2.  The one definition of a
-// particle's column for the push, the sort's keys, the appended particles and
-// the adjoint: an FP32 logarithm guesses the column, the series in y gives the
-// offset to a few 1e-16 relative to r (the 30-instruction FP64 logarithm and its
-// division: 40 pipe slots against about 10), and one step to the neighbour
-// column mends a guess next to an edge.
+// the grid are reported with an offset of 1/2.  The definition that a context's
+// push, sort keys, appended particles and adjoint share: an FP32 logarithm guesses
+// the column, the series in y gives the offset to a few 1e-16 relative to r (the
+// 30-instruction FP64 logarithm and its division: 40 pipe slots against about 10),
+// and one step to the neighbour column mends a guess next to an edge.  The guess's
+// roundings are spelled out: a contraction in one kernel and not in another could
+// put a particle at an edge into different cells for the push and the sort.
+// Contexts without the table and the sort without a context take the logarithm, as
+// grpic_deposit and the diagnostics do; there a particle within rounding of an edge
+// can count to the neighbour column (its weights are continuous across the edge).
 struct ColPos {
     int i;
     double f;
@@ -237,7 +241,7 @@ __device__ __forceinline__ ColPos r_column(const GridDev &g, double r)
 {
     ColPos c;
     if (g.rcen) {
-        const int e = (int)floorf((__logf(float_of_pos(r)) - g.ln_rinf) * g.idx1f);
+        const int e = (int)floorf(__fmul_rn(__fsub_rn(__logf(float_of_pos(r)), g.ln_rinf), g.idx1f));
         c.i = e;
         c.f = 0.5;
         if (e >= -NG && e < g.nr + NG) {

@@ -41,12 +41,11 @@ namespace {
 struct Push64Args {
     GridDev g;
     double dt;
-    double idt, m_i2dt;  // 1 / dt, -1 / (2 dt)
     int n_iter;
     int pairs;           // the correctors before the last may run in pairs
     float hf;            // dt / 2
     df a_df, a2_df, dt_df;
-    double qm[4], qw[4];
+    double qm[4];
     double qdt[4], wr[4], wp[4];  // q dt / (2 m); -q w / (2 dt), q w / dt
     int massive[4];
     int64_t n;
@@ -610,8 +609,7 @@ static Push64Args push64_args(grpic_ctx *ctx, const grpic_particles *in, grpic_p
     Push64Args A;
     A.g = ctx->g;
     A.dt = ctx->prm.dt;
-    A.idt = 1.0 / ctx->prm.dt;
-    A.m_i2dt = -0.5 / ctx->prm.dt;
+    const double idt = 1.0 / ctx->prm.dt, m_i2dt = -0.5 / ctx->prm.dt;
     A.n_iter = ctx->prm.n_push_iter;
     A.pairs = A.n_iter >= 2 && A.dt <= PAIR_MAX_DT;
     A.hf = (float)(0.5 * A.dt);
@@ -620,11 +618,10 @@ static Push64Args push64_args(grpic_ctx *ctx, const grpic_particles *in, grpic_p
     A.dt_df = df_const(A.dt);
     for (int k = 0; k < 4; ++k) {
         A.qm[k] = ctx->prm.q_over_m[k];
-        A.qw[k] = ctx->prm.q_weight[k];
         A.massive[k] = ctx->prm.massive[k];
         A.qdt[k] = 0.5 * A.qm[k] * A.dt;
-        A.wr[k] = A.qw[k] * A.m_i2dt;
-        A.wp[k] = A.qw[k] * A.idt;
+        A.wr[k] = ctx->prm.q_weight[k] * m_i2dt;
+        A.wp[k] = ctx->prm.q_weight[k] * idt;
     }
     A.n = p->n;
     A.d_count = p->d_count;
