@@ -112,7 +112,8 @@ typedef struct {
  * correctors before the last one carry about 44 significant bits of a step's
  * change (double-FP32 pairs) wherever that stays under an eighth of an FP64
  * rounding of the result: dt <= 0.02, dt/2 below 2^-7 r, dt/2 |dphi/dt| below
- * 0.0064, a photon's largest |u_i| at least 2^-40; 53 bits elsewhere.
+ * 0.0064, the largest |u_i| below 2^30 and for a photon at least 2^-30; 53 bits
+ * elsewhere.
  * pusher: the momentum update of charged particles (Sec. 2.2): 0 the
  * generalized Boris step (Eqs. boris-plus-minus .. boris-scheme, the
  * default), 1 Vay's update in the FIDO frame (the paper's alternative; the

@@ -114,23 +114,25 @@ __device__ __forceinline__ void geo_rhs_sc(double a, double a2, double m2a2, dou
 // of dt/2 times the angular velocity or the inverse radius, and the change is of that
 // order of the value.  They run where the square of both is below 2^-14
 // (PAIR_MAX_ANGLE, PAIR_MAX_RADIAL; eps times it is then under an eighth of an FP64
-// rounding of the value), dt is at most PAIR_MAX_DT, and a photon's momentum leaves
-// its square FP32's range (PAIR_MIN_U: a massless right-hand side scales with u, a
-// massive one has the 1 of 1 + u^2), and in FP64 elsewhere: next to the axis and on
-// coarse grids.  Per particle, so that a result does not depend on the warp's other
-// lanes.  Measured over 9 seeds of eight cases, 128^2 to 512^2: every output as far
-// from 64 bits' value as with FP64 correctors, to 1 %.
+// rounding of the value), dt is at most PAIR_MAX_DT, and the low words of u^2 and of
+// its inverse stay in FP32's range (PAIR_MAX_U; PAIR_MIN_U for photons: a massless
+// right-hand side scales with u, a massive one has the 1 of 1 + u^2), and in FP64
+// elsewhere: next to the axis and on coarse grids.  Per particle, so that a result
+// does not depend on the warp's other lanes.  Measured over 9 seeds of eight cases,
+// 128^2 to 512^2: every output as far from 64 bits' value as with FP64 correctors, to
+// 1 %.
 constexpr float PAIR_MAX_ANGLE = 0.0064f;      // of dt/2 |dphi/dt|
 constexpr float PAIR_MAX_RADIAL = 0.0078125f;  // of dt/2 / r
 constexpr double PAIR_MAX_DT = 0.02;
-constexpr int PAIR_MIN_U = 0x3d700000;         // of a photon's largest |u_i|: 2^-40 (high word)
+constexpr int PAIR_MIN_U = 0x3e100000;         // of the largest |u_i|: 2^-30, 2^30 (high words)
+constexpr int PAIR_MAX_U = 0x41d00000;
 
 __device__ __forceinline__ bool pairs_hold(float hf, double xp, double r, bool massive, const double u[3])
 {
     const int top = max(max(__double2hiint(u[0]) & 0x7fffffff, __double2hiint(u[1]) & 0x7fffffff),
                         __double2hiint(u[2]) & 0x7fffffff);
     return hf * float_of_pos(fabs(xp)) < PAIR_MAX_ANGLE && hf < PAIR_MAX_RADIAL * float_of_pos(r) &&
-           (massive || top >= PAIR_MIN_U);
+           (massive || top >= PAIR_MIN_U) && top < PAIR_MAX_U;
 }
 
 struct RhsDf {
