@@ -54,11 +54,11 @@ B0 = 1.0
 # capture of a smaller case of the same workload (same spin, radial range and
 # island fraction), and scaled to a launch by the number of particles.
 PUSH64_FP64_FLOP = 554.2    # FP64 push, 512^2 x 64 ppc split monopole (its early correctors run in FP32 pairs)
-PUSH64_DRAM_B = 95.3        # the same capture: DRAM bytes per particle (read + write)
-PUSH32_FP32_FLOP = 557.1    # FP32-form push, 1024^2 x 64 ppc split monopole
+PUSH64_DRAM_B = 95.4        # the same capture: DRAM bytes per particle (read + write)
+PUSH32_FP32_FLOP = 557.7    # FP32-form push, 1024^2 x 64 ppc split monopole
 # the same capture: instructions issued per particle (warp instructions x 32)
 # and DRAM bytes per particle (read + write)
-PUSH32_INST = 1020.1
+PUSH32_INST = 1021.5
 PUSH32_DRAM_B = 66.8
 # batched 1D lines, b1_kernel with the cascade running (256 lines x 4096 cells):
 # instructions issued per particle-step (warp instructions x 32) and DRAM
@@ -75,8 +75,8 @@ B1_ALG_B = 2 * 28
 # Vay's update (1024^2 x 64 ppc), the FP64 push with the cubic shape (512^2 x
 # 64 ppc), the FP64 push with photon emission and conversion decisions (512^2
 # x 16 ppc, Wald a = 0.99, B0 = 500)
-VAY32_FP32_FLOP = 614.8
-VAY32_INST = 1095.7
+VAY32_FP32_FLOP = 615.3
+VAY32_INST = 1097.1
 CUBIC64_FP64_FLOP = 984.3
 RAD64_FP64_FLOP = 644.3
 VAY_COUNT = "ncu SASS counters, FP32-form push with Vay's update, 1024^2 x 64 ppc"
