@@ -175,6 +175,7 @@ grpic_status prepare_push(grpic_ctx *ctx, grpic_fields *f, int32_t *cnt9, cudaSt
 grpic_status ensure_particle_scratch(grpic_ctx *ctx, int64_t n)
 {
     if (n <= ctx->keys_cap) return GRPIC_OK;
+    ctx->keys_valid = ctx->hist_valid = 0;  // the keys go with their buffer, also where the new one fails
     if (ctx->d_keys) cudaFree(ctx->d_keys);
     if (ctx->d_perm) cudaFree(ctx->d_perm);
     ctx->d_keys = nullptr;
