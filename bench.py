@@ -78,7 +78,7 @@ B1_ALG_B = 2 * 28
 VAY32_FP32_FLOP = 615.3
 VAY32_INST = 1097.1
 CUBIC64_FP64_FLOP = 984.3
-RAD64_FP64_FLOP = 644.3
+RAD64_FP64_FLOP = 645.3
 VAY_COUNT = "ncu SASS counters, FP32-form push with Vay's update, 1024^2 x 64 ppc"
 CUBIC_COUNT = "ncu SASS counters, FP64 push with the cubic shape, 512^2 x 64 ppc"
 RAD_COUNT = "ncu SASS counters, FP64 push with emission/conversion decisions, 512^2 x 16 ppc"

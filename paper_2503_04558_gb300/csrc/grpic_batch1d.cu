@@ -21,11 +21,14 @@
 // the first's and the children follow in parent order: the same line state
 // as one CTA would leave, up to the rounding of the current's sum.
 //
-// Bound by instruction issue (70 % of the slots, about 910 instructions per
-// particle-step before any photon).  20 steps of 512 lines x 4096 cells, 1.03e7
-// particles: 10.26 -> 9.41 ms with the currents' sums in 32-bit words, divisions
-// by tabulated values through their inverses (the same results bit for bit), the
-// ranks by ballots and the emission's FP32 screen on hardware reciprocals.
+// Bound by instruction issue on the SM of the longest line (70 % of the slots,
+// about 910 instructions per particle-step before any photon).  With one CTA per
+// line the launch ends no earlier than that line: of 512 lines x 4096 cells, 1.03e7
+// particles, the longest has 99 190 against 67 940 per SM, so the SMs together are at
+// most 68 % used.  20 steps of those: 10.26 -> 9.41 ms with the currents' sums in
+// 32-bit words, divisions by tabulated values through their inverses (the same
+// results bit for bit), the ranks by ballots and the emission's FP32 screen on
+// hardware reciprocals.
 #include "grpic_geo.cuh"
 #include "grpic_philox.cuh"
 
